@@ -135,7 +135,13 @@ void build_ntab(sl_ntab& t, int n, int basis, int dim, bool mixed2d, TableBufs& 
   for (int mask = 0; mask < 4; ++mask)
     for (int soft = 0; soft < 2; ++soft) {
       const FitOps& f = t.fit[mask][soft];
-      t.table_off[mask][soft][0] = B.put(f.Cpinv, 1);
+      // 2D: row of C first ([k][node]), so that the threads of an element (one per node) read
+      // consecutive values
+      std::vector<double> cp = f.Cpinv;
+      if (dim == 2 && !cp.empty())
+        for (int q = 0; q < f.nd; ++q)
+          for (int k = 0; k < f.m; ++k) cp[(size_t)k * f.nd + q] = f.Cpinv[(size_t)q * f.m + k];
+      t.table_off[mask][soft][0] = B.put(cp, 1);
       t.table_off[mask][soft][1] = B.put(f.S, 1);
       t.table_off[mask][soft][2] = B.put(f.SCt, 1);
     }
@@ -307,7 +313,7 @@ sl_status finish_uniform(sl_ctx* c) {
   }
   alias_ntab(c);
   const size_t work_bytes = M.dim != 2 ? 0
-                            : c->precision == SL_FP64 ? work2d_doubles(c->nel, c->n) * sizeof(double)
+                            : c->precision == SL_FP64 ? work2d_doubles(c->nvals, c->nel, 4 * c->n) * sizeof(double)
                                                       : work2m_floats(c->nel, c->n) * sizeof(float);
   return alloc_upload(c, B, work_bytes);
 }
@@ -340,7 +346,7 @@ sl_status finish_mapped(sl_ctx* c, const std::vector<uint16_t>& prob = {}) {
     c->bucket_count[n] = pos - c->bucket_start[n];
   }
   const size_t work_bytes = c->precision == SL_FP64
-                                ? (size_t)(c->nvals + nel * (4 * NMAX + 8)) * sizeof(double)
+                                ? (size_t)work2d_doubles(c->nvals, nel, 4 * NMAX) * sizeof(double)
                                 : (size_t)(c->nvals + nel * (4 * NMAX + WORK2M_FACE + WORK2M_ELEM)) * sizeof(float);
   sl_status st = alloc_upload(c, B, work_bytes);
   if (st != SL_OK) return st;
@@ -628,7 +634,17 @@ sl_status step2d_general(sl_ctx* c, StepParams P, const sl_velocity* vel, double
         Tables1D tb{T + N.off_xi, T + N.off_w, T + N.off_lam, T + N.off_l0, T + N.off_l1,
                     T + off[0],   T + off[1],  T + off[2],    T + c->off_rules};
         double* W = c->d_work;
-        Work2D w{W, W + c->nvals, W + c->nvals + nel * ts};
+        Work2D w{W, W + c->nvals, W + c->nvals + nel * ts, (uint8_t*)(W + c->nvals + nel * (ts + 8))};
+        // one displacement for all elements: phase 1 as shared operators (the backtracked values of
+        // eq. 4.11 and meshes of several node counts or steps take the general kernel)
+        if (phase == 1 && vel->kind == SL_VEL_CONST && !c->mapped && opt->bvalue == SL_BV_INTERP) {
+          Shift2D& S = c->shift2;
+          if (!S.valid || S.a != vel->p[0] || S.b != vel->p[1] || S.dt != dt || S.rk != opt->rk_order)
+            build_shift2d(N.b, vel->p[0], vel->p[1], dt, hx, hy, opt->rk_order, S);
+          launch_step2d_f64_shift(n, S, P, count, (const double*)in, w, c->stream);
+          SL_CUDA(c, cudaGetLastError());
+          continue;
+        }
         launch_step2d_f64(phase, n, P, tb, map, count, (const double*)in, (double*)out, w, c->d_status, c->stream);
         SL_CUDA(c, cudaGetLastError());
       } else {

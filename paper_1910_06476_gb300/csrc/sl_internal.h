@@ -63,7 +63,7 @@ struct Tables1D {                         // device pointers into one table buff
   const double* lam;
   const double* l0;
   const double* l1;
-  const double* Cpinv;                   // [n][m] for the active row set
+  const double* Cpinv;                   // active row set: [n][m] in 1D, [m][n^2] in 2D
   const double* S;                       // [n][n]
   const double* SCt;                     // [n][m]
   const double* rules;                   // [NMAX + 1][3][NMAX] xi, lam, w of every node count
@@ -119,14 +119,37 @@ struct Map2D {
 struct Work2D {                          // FP64 workspace between the two phases
   double* phihat;                        // same layout as the state
   double* traces;                        // [nel][tstride]   faces W, E, S, N at the tangential nodes
-  double* fluxes;                        // [nel][4][2]      outflow (mass, energy) flux per face
+  double* fluxes;                        // [nel][4][2]      (mass, energy) flux per face: outflow, and the
+                                         //                  ghost's inflow through a domain face
+  uint8_t* side;                         // [nel][tstride]   upwind side of each face point at t^{n+1}: 0 own,
+                                         //                  1 neighbour or ghost, 2 tie
 };
 
 // 2D FP64 step: phase 1 (remap, traces, outflow fluxes) of every launch must run before any
-// phase 2 (interface values, targets, fit); count = CTAs (elements) of the launch
+// phase 2 (interface values, targets, fit); count = elements of the launch
 void launch_step2d_f64(int phase, int n, const StepParams& p, const Tables1D& tb, const Map2D& m, int64_t count,
                        const double* in, double* out, const Work2D& w, unsigned* status, cudaStream_t s);
-inline int64_t work2d_doubles(int64_t nel, int n) { return nel * (int64_t)(n * n + 4 * n + 8); }
+// doubles of the workspace for nvals values and nel elements of ts face points (sides: one byte each)
+inline int64_t work2d_doubles(int64_t nvals, int64_t nel, int ts) { return nvals + nel * (ts + 8) + (nel * ts + 7) / 8; }
+
+// Operators of a constant-velocity FP64 step on a mesh of one node count (every element sees the same
+// displacement), built on the host in double (ops_shift.cpp) and passed to the kernels by value.  Stages
+// are the distinct stage times of the RK scheme; stage 0 is t^n.
+struct Shift2D {
+  bool valid = false;
+  double a = 0, b = 0, dt = 0;
+  int rk = 0, nst = 0;
+  double Rx[NMAX * NMAX], Ry[NMAX * NMAX];   // remap: [l][q] = h_q(xi_l - shift)
+  double bx[3][NMAX], by[3][NMAX];           // basis at the feet of the x- / y-outflow face
+  double wx[3][NMAX], wy[3][NMAX];           // b_s sum_q w_q (basis at the tangential foot of point q)
+  double Bx[2][NMAX * NMAX], By[2][NMAX * NMAX];   // [point][m]: that basis, stages 1 and 2
+  double bs[3];                              // summed RK weights per distinct stage
+  double l0[NMAX], l1[NMAX], w[NMAX];
+};
+void build_shift2d(const Basis1D& B, double a, double b, double dt, double hx, double hy, int rk, Shift2D& S);
+// phase 1 of the constant-velocity step (phase 2 is that of launch_step2d_f64)
+void launch_step2d_f64_shift(int n, const Shift2D& h, const StepParams& p, int64_t count, const double* in,
+                             const Work2D& w, cudaStream_t s);
 
 // Extra parameters of the 2D mixed-precision kernels (float tables and scalars), by value
 struct Mixed2DExtra {
@@ -310,6 +333,7 @@ struct sl_ctx {
   sl::ProbGeom* d_geo_run = nullptr;     // per-step geometry of a batch run, [nsteps][nprob]
   size_t geo_run_cap = 0;
   const sl::ProbGeom* geo_override = nullptr;
+  sl::Shift2D shift2{};                  // operators of the last constant-velocity FP64 step
   // cached shared operator of the mixed 2D constant-velocity path
   bool m2c_valid = false;
   double m2c_a = 0, m2c_b = 0, m2c_dt = 0;
