@@ -30,9 +30,10 @@
 //     CTA's slots, the flux at stage time t^n is a plain trace;
 //   - sums over an element go through shared memory, one thread per row, instead of a butterfly in which
 //     every lane adds; maxima compare the high words of the values as integers.
-// Measured (one GB300): swirl, 128 x 96 elements of n = 8, every constraint: 4.99 -> 1.38 ms per step against
+// Measured (one GB300): swirl, 128 x 96 elements of n = 8, every constraint: 4.99 -> 1.29 ms per step against
 // one element per CTA with FP64 sines, a FP64 preconditioner and 5-6 FP64 residuals per solve (3030 -> 530
-// FP64 instructions per node in phase 1, pipe 84 % busy); rotation, 66 x 61, n = 8: 0.87 -> 0.32 ms.
+// FP64 instructions per node in phase 1, pipe 84 % busy; phase 2 waits on the few elements whose energy
+// iteration runs to its cap); rotation, 66 x 61, n = 8: 0.87 -> 0.30 ms.
 #include <cfloat>
 
 #include "k_map2d.cuh"
@@ -101,7 +102,9 @@ __device__ __forceinline__ int nb_index(int kx, int ky, const int* bc, int ex, i
   return jy * kx + jx;
 }
 
-template <int NN>
+// PHASE 2 needs neither positions nor velocities: one thread sets up a slot, and each of its FP64
+// instructions holds a scheduler's pipe for 64 cycles
+template <int NN, int PHASE>
 __device__ __forceinline__ void geo_setup(const StepParams& P, const Map2D& M, int64_t k, int64_t count, Geo& G) {
   G.valid = k < count;
   for (int f = 0; f < 4; ++f) { G.nb[f] = -1; G.nq[f] = 0; }
@@ -112,6 +115,7 @@ __device__ __forceinline__ void geo_setup(const StepParams& P, const Map2D& M, i
   int kx = P.kx, ky = P.ky, bc[4] = {P.bc[0], P.bc[1], P.bc[2], P.bc[3]};
   double X0 = P.x0, Y0 = P.y0;
   G.hx = P.hx; G.hy = P.hy; G.t = P.t; G.dt = P.dt; G.ghost = P.ghost;
+  G.lam = P.lam;
   if (M.geo) {
     const ProbGeom& Q = M.geo[M.prob[G.g]];
     kx = Q.kx; ky = Q.ky;
@@ -119,20 +123,23 @@ __device__ __forceinline__ void geo_setup(const StepParams& P, const Map2D& M, i
     X0 = Q.x0; Y0 = Q.y0;
     G.hx = Q.hx; G.hy = Q.hy; G.t = Q.t; G.dt = Q.dt; G.ghost = Q.ghost;
     G.gb = Q.gbase;
+    G.lam = G.dt / (G.hx * G.hy);
   }
   const int e = (int)(G.g - G.gb);
   G.ex = e % kx;
   G.ey = e / kx;
   G.base = M.off ? M.off[G.g] : G.g * (NN * NN);
-  G.lam = G.dt / (G.hx * G.hy);
-  G.x0 = X0 + G.ex * G.hx;
-  G.y0 = Y0 + G.ey * G.hy;
+  if (PHASE == 1) {
+    G.x0 = X0 + G.ex * G.hx;
+    G.y0 = Y0 + G.ey * G.hy;
+  }
   for (int f = 0; f < 4; ++f) {
     G.nb[f] = nb_index(kx, ky, bc, G.ex, G.ey, f);
     // a face shared with an element of more nodes takes the rule of the finer side, so that both
     // elements integrate the same points (the flux telescopes)
     G.nq[f] = G.nb[f] < 0 ? NN : max(NN, order_of<NN>(M, G.gb + G.nb[f]));
   }
+  if (PHASE == 2) return;
   if (P.vel_kind == SL_VEL_ROTATION) {
     G.kx = -P.vp[0] * G.hy / G.hx;
     G.ky = P.vp[0] * G.hx / G.hy;
@@ -431,7 +438,7 @@ struct Shape {
   static constexpr int NPD = (NN + 1) & ~1;                // row stride of double tables (16-byte rows)
   static constexpr int NPF = (NN + 3) & ~3;                // row stride of float tables
   // resident CTAs asked of the compiler: one CTA's FP32 passes and barriers hide behind another's FP64 work
-  static constexpr int MINB = NN <= 10 ? 2 : 1, MINB2 = 2;
+  static constexpr int MINB = NN <= 10 ? 2 : 1, MINB2 = NN <= 10 ? 4 : 3;
 };
 
 __device__ __forceinline__ double hi_value(int h) { return __hiloint2double(h, 0); }
@@ -480,7 +487,7 @@ __global__ void __launch_bounds__(Shape<NN>::NTMAX, NOD ? 1 : Shape<NN>::MINB)
     s_lamf[tid] = (float)tb.lam[tid];
   }
   if (tid < slots) {
-    geo_setup<NN>(P, M, (int64_t)blockIdx.x * slots + tid, count, SL[tid].G);
+    geo_setup<NN, 1>(P, M, (int64_t)blockIdx.x * slots + tid, count, SL[tid].G);
     for (int k = 0; k < 3; ++k) { SL[tid].mx[k] = 0; SL[tid].fm[k] = 0; }
   }
   if (tid == 0) s_items = 0;
@@ -857,15 +864,50 @@ struct __align__(16) Slot2 {
   static constexpr int MMAX = 4 * NN + 1;
   double ph[NN * NN], a[NN * NN];           // phihat; energy iteration: w o phi
   double r[MMAX], d[MMAX], ca[MMAX];
-  double rs[3][NN], tot[3];                 // sums over the element: rows, totals
-  double netm, nete;
+  double rs[2][NN], tot[2];                 // sums over the element: rows, totals
+  double netm, nete, Et, gamma, s;          // net fluxes; energy target, miss and step along q
   Geo G;
   int rows[4];                              // faces with a non-zero residual
+  int on, feasible, mx, ht;                 // energy iteration: running, maximum (high word), tolerance
 };
 
 template <int NN>
 inline size_t smem2(int slots) {
   return (size_t)slots * (sizeof(Slot2<NN>) + (size_t)3 * NN * NN * sizeof(double));
+}
+
+// the neighbour's trace across a p-nonconforming face, out of line: its 2 x 17 products in registers would
+// set the register count of the whole kernel
+static __device__ __noinline__ double interp_far(const double* rules, int nn, const double* tr, double z) {
+  return interp_rule(rules, nn, tr, z);
+}
+
+// sum of NN values a stride apart, in two interleaved chains (fixed order)
+template <int NN>
+__device__ __forceinline__ double chain_sum(const double* v) {
+  double a = v[0], b = NN > 1 ? v[1] : 0.0;
+#pragma unroll
+  for (int k = 2; k < NN; ++k) (k & 1 ? b : a) += v[k];
+  return a + b;
+}
+
+// Sums of nq quantities buf[slot][quantity][node] over the elements that are on, in a fixed order: one thread
+// per row, then one per quantity.  Called by every thread of the CTA; not inlined, it is used several times.
+template <int NN>
+__device__ __noinline__ void slot_sums(const double* buf, Slot2<NN>* SL, int slots, int nq) {
+  constexpr int ND = NN * NN;
+  const int tid = threadIdx.x, nt = blockDim.x;
+  __syncthreads();
+  for (int idx = tid; idx < slots * nq * NN; idx += nt) {
+    const int s = idx / (nq * NN), q = (idx / NN) % nq, row = idx % NN;
+    if (SL[s].on) SL[s].rs[q][row] = chain_sum<NN>(buf + ((size_t)s * 3 + q) * ND + row * NN);
+  }
+  __syncthreads();
+  for (int idx = tid; idx < slots * nq; idx += nt) {
+    const int s = idx / nq, q = idx % nq;
+    if (SL[s].on) SL[s].tot[q] = chain_sum<NN>(SL[s].rs[q]);
+  }
+  __syncthreads();
 }
 
 template <int NN>
@@ -883,8 +925,10 @@ __global__ void __launch_bounds__(Shape<NN>::NTMAX, Shape<NN>::MINB2)
     s_l0[tid] = tb.l0[tid]; s_l1[tid] = tb.l1[tid];
   }
   if (tid < slots) {
-    geo_setup<NN>(P, M, (int64_t)blockIdx.x * slots + tid, count, SL[tid].G);
+    geo_setup<NN, 2>(P, M, (int64_t)blockIdx.x * slots + tid, count, SL[tid].G);
     for (int f = 0; f < 4; ++f) SL[tid].rows[f] = 0;
+    SL[tid].on = SL[tid].G.valid;
+    SL[tid].mx = 0;
   }
   __syncthreads();
   const int slot = tid / ND < slots ? tid / ND : 0;
@@ -903,29 +947,8 @@ __global__ void __launch_bounds__(Shape<NN>::NTMAX, Shape<NN>::MINB2)
   const bool mass = (P.cons & SL_C_MASS) != 0, energy = (P.cons & SL_C_ENERGY) != 0;
   const bool hard = P.fit == SL_FIT_HARD;
   const int nb_rows = bnd ? 4 * NN : 0, m = P.m;
-  // sums of up to three quantities over each element, in a fixed order (rows, then their sum)
   double* mine = buf + (size_t)slot * 3 * ND;
   auto put = [&](int q, double v) { if (part) mine[q * ND + nd] = v; };
-  auto sums = [&](int nq, bool maxi) {
-    __syncthreads();
-    for (int idx = tid; idx < slots * nq * NN; idx += nt) {
-      const int s = idx / (nq * NN), q = (idx / NN) % nq, row = idx % NN;
-      const double* v = buf + ((size_t)s * 3 + q) * ND + row * NN;
-      double acc = v[0];
-#pragma unroll
-      for (int k = 1; k < NN; ++k) acc = maxi ? fmax(acc, v[k]) : acc + v[k];
-      SL[s].rs[q][row] = acc;
-    }
-    __syncthreads();
-    for (int idx = tid; idx < slots * nq; idx += nt) {
-      const int s = idx / nq, q = idx % nq;
-      double acc = SL[s].rs[q][0];
-#pragma unroll
-      for (int k = 1; k < NN; ++k) acc = maxi ? fmax(acc, SL[s].rs[q][k]) : acc + SL[s].rs[q][k];
-      SL[s].tot[q] = acc;
-    }
-    __syncthreads();
-  };
   // upwinded interface values (rows W, E, S, N at the tangential nodes); residual d - C phihat
   if (bnd)
     for (int idx = tid; idx < slots * 4 * NN; idx += nt) {
@@ -941,7 +964,7 @@ __global__ void __launch_bounds__(Shape<NN>::NTMAX, Shape<NN>::MINB2)
         if (nb >= 0) {                         // the neighbour's trace (opposite face) at this face point
           const int nn = order_of<NN>(M, T.G.gb + nb);
           const double* tr = W.traces + (T.G.gb + nb) * M.tstride + (f ^ 1) * nn;
-          other = nn == NN ? tr[q] : interp_rule(tb.rules, nn, tr, s_xi[q]);
+          other = nn == NN ? tr[q] : interp_far(tb.rules, nn, tr, s_xi[q]);
         }
         if (side == 1) val = other;
         else if (nb >= 0) val = 0.5 * (own + other);
@@ -960,8 +983,8 @@ __global__ void __launch_bounds__(Shape<NN>::NTMAX, Shape<NN>::MINB2)
       T.r[t] = rr;
       if (!(rr == 0.0)) T.rows[f] = 1;         // (any thread: the same value)
     }
-  // mass and energy targets (reference measure): net flux from the faces in order
-  double Et = 0.0;
+  // mass and energy targets (reference measure): net flux from the faces in order; scalars by one thread per
+  // slot (an instruction of every thread costs the pipe eight times as much)
   if (mass || energy) {
     for (int idx = tid; idx < 2 * slots; idx += nt) {
       Slot2<NN>& T = SL[idx >> 1];
@@ -974,16 +997,14 @@ __global__ void __launch_bounds__(Shape<NN>::NTMAX, Shape<NN>::MINB2)
       }
       (k ? T.nete : T.netm) = net;
     }
-    put(0, w2 * (phn - ph));                   // M^n - M(phihat)
-    if (energy || !hard) put(1, w2 * phn * phn);
-    if (!hard) put(2, w2 * phn);
-    sums(hard ? (energy ? 2 : 1) : 3, false);
-    const double lam = S.G.lam;
-    if (mass && nd == 0 && part) {
-      S.r[nb_rows] = S.tot[0] - lam * S.netm;
-      S.d[nb_rows] = S.tot[2] - lam * S.netm;  // read by the soft fit only
+    put(0, hard ? w2 * (phn - ph) : w2 * phn); // hard: M^n - M(phihat)
+    if (energy) put(1, w2 * phn * phn);
+    slot_sums<NN>(buf, SL, slots, energy ? 2 : 1);
+    if (tid < slots && SL[tid].G.valid) {
+      Slot2<NN>& T = SL[tid];
+      if (mass) T.r[nb_rows] = T.d[nb_rows] = T.tot[0] - T.G.lam * T.netm;   // residual (hard), target (soft)
+      if (energy) T.Et = T.tot[1] - T.G.lam * T.nete;
     }
-    Et = S.tot[1] - lam * S.nete;
   }
   __syncthreads();
   // linear constrained fit; a face whose rows all vanish (outflow: own trace) adds nothing
@@ -1009,76 +1030,101 @@ __global__ void __launch_bounds__(Shape<NN>::NTMAX, Shape<NN>::MINB2)
   bool ok = true;
   if (energy) {
     put(0, w2 * phL * phL);
-    sums(1, false);
-    const double EL = S.tot[0];
-    const double gamma = EL - Et;
-    const bool apply = part && fabs(gamma) > ENERGY_SKIP_RTOL * fmax(fabs(Et), EL);
-    if (__syncthreads_or(apply)) {
-      put(0, fabs(ph));
-      sums(1, true);
-      const double tol = P.picard_rtol * fmax(S.tot[0], 1e-300);
-      bool conv = false, feasible = true, on = apply;          // equal in every thread of a slot
+    slot_sums<NN>(buf, SL, slots, 1);
+    bool run = false;
+    if (tid < slots) {
+      Slot2<NN>& T = SL[tid];
+      const double EL = T.tot[0];
+      T.gamma = EL - T.Et;
+      run = T.G.valid && fabs(T.gamma) > ENERGY_SKIP_RTOL * fmax(fabs(T.Et), EL);
+      T.on = run;
+    }
+    if (__syncthreads_or(run)) {
+      // Few elements of a CTA iterate, some of them up to the cap, and set the tail of the launch: only their
+      // threads work, and the scalars (a square root and a division) are formed by one thread per slot.
+      // Equal in every thread of a slot:
+      bool on = part && S.on, conv = false;
+      const bool apply = on;
+      if (on) atomicMax(&S.mx, hi_abs(ph));
+      __syncthreads();
+      if (tid < slots) SL[tid].ht = hi_abs(P.picard_rtol * fmax(hi_value(SL[tid].mx), 1e-300));
       for (int it = 0; it < P.picard_cap; ++it) {
-        const double a = w2 * cur;
-        double q = 0.0;
-        if (on) S.a[nd] = a;
+        double a = 0.0, q = 0.0;
+        if (on) {
+          a = w2 * cur;
+          S.a[nd] = a;
+          if (mass) put(0, w2 * a);
+        }
+        __syncthreads();
         if (hard) {
-          // C a: boundary rows (traces of a), then the mass row
-          put(0, w2 * a);
-          sums(1, false);
-          if (on && mass && nd == 0) S.ca[nb_rows] = S.tot[0];
-          if (bnd)
-            for (int idx = tid; idx < slots * 4 * NN; idx += nt) {
-              Slot2<NN>& T = SL[idx / (4 * NN)];
-              const int t = idx % (4 * NN), f = t / NN, qq = t % NN;
+          // C a: boundary rows (traces of a), the mass row's row sums
+          for (int idx = tid; idx < slots * 5 * NN; idx += nt) {
+            Slot2<NN>& T = SL[idx / (5 * NN)];
+            if (!T.on) continue;
+            const int t = idx % (5 * NN), f = t / NN, qq = t % NN;
+            if (f == 4) {
+              if (mass) T.rs[0][qq] = chain_sum<NN>(buf + (size_t)(idx / (5 * NN)) * 3 * ND + qq * NN);
+            } else if (bnd) {
               const double* L = (f == 1 || f == 3) ? s_l1 : s_l0;
               double acc = 0.0;
 #pragma unroll
               for (int k = 0; k < NN; ++k) acc += (f < 2 ? T.a[qq * NN + k] : T.a[k * NN + qq]) * L[k];
               T.ca[t] = acc;
             }
+          }
           __syncthreads();
+          // q = a - C+ (C a), the rows in order (where the two roots of the energy equation meet, whether the
+          // iteration settles below the tolerance hangs on the rounding of this sum)
           if (on) {
             double acc = a;
-            for (int k = 0; k < m; ++k) acc -= tb.Cpinv[(size_t)k * ND + nd] * S.ca[k];
+#pragma unroll 8
+            for (int k = 0; k < nb_rows; ++k) acc -= tb.Cpinv[(size_t)k * ND + nd] * S.ca[k];
+            if (mass) acc -= tb.Cpinv[(size_t)nb_rows * ND + nd] * chain_sum<NN>(S.rs[0]);
             q = acc;
+            put(0, w2 * phL * q);
+            put(1, w2 * q * q);
           }
-          put(0, w2 * phL * q);
-          put(1, w2 * q * q);
-          sums(2, false);
-          const double alpha = S.tot[0], beta = S.tot[1];
-          double s;
-          if (beta <= 0.0) { s = 0.0; feasible = gamma <= 0.0; }
-          else {
-            const double disc = alpha * alpha - beta * gamma;
-            if (disc < 0.0) { s = -alpha / beta; feasible = false; }
-            else {
-              const double root = sqrt(disc);
-              const double den = alpha + (alpha >= 0.0 ? root : -root);
-              s = den == 0.0 ? 0.0 : -gamma / den;
-              feasible = true;
-            }
-          }
-          q = phL + s * q;
-        } else {
-          __syncthreads();
-          if (on) {
-            double acc = 0.0;
-            for (int k = 0; k < ND; ++k) acc += tb.S[(size_t)nd * ND + k] * S.a[k];
-            q = acc;
-          }
+        } else if (on) {
+          double acc = 0.0;
+          for (int k = 0; k < ND; ++k) acc += tb.S[(size_t)nd * ND + k] * S.a[k];
+          q = acc;
           put(0, a * phL);
           put(1, a * q);
-          sums(2, false);
-          const double s = (Et - S.tot[0]) / (1.0 + S.tot[1]);
-          q = phL + s * q;
-          feasible = true;
         }
-        put(0, fabs(q - cur));
-        sums(1, true);
+        slot_sums<NN>(buf, SL, slots, 2);
+        if (tid < slots && SL[tid].on) {
+          Slot2<NN>& T = SL[tid];
+          const double alpha = T.tot[0], beta = T.tot[1], gamma = T.gamma;
+          T.mx = 0;
+          T.feasible = 1;
+          if (!hard) {
+            T.s = (T.Et - alpha) / (1.0 + beta);
+          } else if (beta <= 0.0) {
+            T.s = 0.0;
+            T.feasible = gamma <= 0.0;
+          } else {
+            const double disc = alpha * alpha - beta * gamma;
+            if (disc < 0.0) {
+              T.s = -alpha / beta;
+              T.feasible = 0;
+            } else {
+              const double root = sqrt(disc);
+              const double den = alpha + (alpha >= 0.0 ? root : -root);
+              T.s = den == 0.0 ? 0.0 : -gamma / den;
+            }
+          }
+        }
+        __syncthreads();
         if (on) {
-          cur = q;
-          if (S.tot[0] < tol) { conv = feasible; on = false; }
+          const double nv = phL + S.s * q;
+          atomicMax(&S.mx, hi_abs(nv - cur));
+          cur = nv;
+        }
+        __syncthreads();
+        if (on && S.mx < S.ht) {               // (high words: below the tolerance for certain)
+          conv = S.feasible;
+          on = false;
+          if (nd == 0) S.on = 0;
         }
         if (!__syncthreads_or(on)) break;
       }
@@ -1131,8 +1177,8 @@ void launch_n(int phase, const StepParams& p, const Tables1D& tb, const Map2D& m
 // thread j takes row j of phi^n through R_x, then column j of the result through R_y.  Operator entries are
 // the same for every thread, so they come from the parameter bank as DFMA operands; entries that differ by
 // thread sit in shared memory.  About 2 n + 10 FP64 instructions per node, where the per-element solve takes
-// a few hundred: 512 x 512 elements of n = 9 with the mass row, both phases, 52.2 -> 3.44 ms per step (this
-// kernel: 29 FP64 instructions per node, pipe 79 % busy).
+// a few hundred: 512 x 512 elements of n = 9 with the mass row, both phases, 52.2 -> 2.77 ms per step (this
+// kernel: 29 FP64 instructions per node, pipe 79 % busy; phase 2: 31, 72 %).
 template <int NN>
 struct ShiftOps {
   double Rx[NN * NN], Ry[NN * NN];          // remap: R[l][q] = h_q(xi_l - shift)

@@ -2,6 +2,7 @@
 // displacement, so the remap (eq. 4.9, 5.4) and the flux feet (eq. remap_mass, remap_energy) are fixed
 // matrices.  Differences are formed as (z0 - xi_k) + dz in reference coordinates, so the displacement is
 // not rounded to the element's physical position.  Double arithmetic, O(n^3) operations (microseconds).
+#include <algorithm>
 #include <cmath>
 
 #include "sl_internal.h"
@@ -25,6 +26,25 @@ const double ds_c[5][3] = {{}, {0.0}, {0.0, 1.0}, {0.0, 0.5, 1.0}, {0.0, 0.5, 1.
 const double ds_b[5][3] = {{}, {1.0}, {0.5, 0.5}, {1.0 / 6, 2.0 / 3, 1.0 / 6}, {1.0 / 6, 2.0 / 3, 1.0 / 6}};
 
 }  // namespace
+
+void build_shift1d(const Basis1D& B, double a, double dt, double h, int rk, Shift1D& S) {
+  const double sx = dt * a / h;                         // displacement in reference units
+  S.nst = ds_n[rk];
+  for (int j = 0; j < B.n; ++j) basis_row(B, B.xi[j], -sx, S.R + j * B.n);
+  for (int s = 0; s < 3; ++s) {
+    S.bs[s] = s < S.nst ? ds_b[rk][s] : 0.0;
+    basis_row(B, a > 0.0 ? 1.0 : 0.0, s < S.nst ? -ds_c[rk][s] * sx : 0.0, S.E[s]);
+  }
+  for (int f = 0; f < 2; ++f) {
+    const std::vector<double>& l = f ? B.l1 : B.l0;
+    std::copy(l.begin(), l.end(), S.L[f]);
+    basis_row(B, f, -sx, S.B[f]);
+  }
+  S.a = a;
+  S.dt = dt;
+  S.rk = rk;
+  S.valid = true;
+}
 
 void build_shift2d(const Basis1D& B, double a, double b, double dt, double hx, double hy, int rk, Shift2D& S) {
   const int n = B.n;

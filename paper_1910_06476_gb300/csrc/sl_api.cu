@@ -746,6 +746,7 @@ sl_status step_dispatch(sl_ctx* c, const void* phi_in, void* phi_out, const sl_v
   for (int i = 0; i < 6; ++i) P.vp[i] = vel->p[i];
   P.t = t;
   P.dt = dt;
+  P.lam = dt / (hx * hy);
   P.rk = opt->rk_order;
   P.cons = opt->constraints;
   P.fit = opt->fit;
@@ -764,7 +765,11 @@ sl_status step_dispatch(sl_ctx* c, const void* phi_in, void* phi_out, const sl_v
   if (M.dim == 1 && c->precision == SL_FP64) {
     Tables1D tb{T + c->off_xi, T + c->off_w, T + c->off_lam, T + c->off_l0, T + c->off_l1,
                 T + off[0], T + off[1], T + off[2]};
-    launch_step1d_f64(c->n, P, tb, (const double*)phi_in, (double*)phi_out, c->d_status, c->stream);
+    // one displacement for all elements: shared operators
+    Shift1D* S = vel->kind == SL_VEL_CONST ? &c->shift1 : nullptr;
+    if (S && (!S->valid || S->a != vel->p[0] || S->dt != dt || S->rk != opt->rk_order))
+      build_shift1d(c->b, vel->p[0], dt, hx, opt->rk_order, *S);
+    launch_step1d_f64(c->n, P, tb, S, c->b.xi.data(), (const double*)phi_in, (double*)phi_out, c->d_status, c->stream);
   } else if (M.dim == 1 && c->precision == SL_MIXED) {
     if (vel->kind != SL_VEL_CONST)
       return fail(c, SL_EUNSUPPORTED, "the 1D mixed path needs a constant velocity (shared operator)");

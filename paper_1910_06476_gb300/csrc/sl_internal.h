@@ -78,6 +78,7 @@ struct StepParams {
   int vel_kind;
   double vp[6];
   double t, dt;
+  double lam;                            // dt / (hx hy)
   int rk;
   unsigned cons;
   int fit;
@@ -90,8 +91,19 @@ struct StepParams {
   int64_t nvals;                         // state values (stride of the nodal components)
 };
 
-void launch_step1d_f64(int n, const StepParams& p, const Tables1D& tb, const double* in,
-                       double* out, unsigned* status, cudaStream_t s);
+// Operators of a constant-velocity 1D FP64 step (ops_shift.cpp): remap [j][i] = h_i(xi_j - shift), basis at
+// the feet of the outflow face per distinct stage time, summed RK weights.
+struct Shift1D {
+  bool valid = false;
+  double a = 0, dt = 0;
+  int rk = 0, nst = 0;
+  double R[NMAX * NMAX], E[3][NMAX], bs[3];
+  double L[2][NMAX], B[2][NMAX];             // basis at the faces, and at their backward feet from t^{n+1}
+};
+void build_shift1d(const Basis1D& B, double a, double dt, double h, int rk, Shift1D& S);
+// h: operators of a constant velocity, else null; xi_host: the nodes
+void launch_step1d_f64(int n, const StepParams& p, const Tables1D& tb, const Shift1D* h, const double* xi_host,
+                       const double* in, double* out, unsigned* status, cudaStream_t s);
 
 // Geometry and step of one problem of a batch (device array); replaces the StepParams fields of
 // the same names for the elements of that problem.
@@ -333,7 +345,8 @@ struct sl_ctx {
   sl::ProbGeom* d_geo_run = nullptr;     // per-step geometry of a batch run, [nsteps][nprob]
   size_t geo_run_cap = 0;
   const sl::ProbGeom* geo_override = nullptr;
-  sl::Shift2D shift2{};                  // operators of the last constant-velocity FP64 step
+  sl::Shift1D shift1{};                  // operators of the last constant-velocity FP64 step
+  sl::Shift2D shift2{};
   // cached shared operator of the mixed 2D constant-velocity path
   bool m2c_valid = false;
   double m2c_a = 0, m2c_b = 0, m2c_dt = 0;

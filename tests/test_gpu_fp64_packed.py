@@ -82,7 +82,7 @@ SHIFT = [
     # kx, ky, n, params, bc, cons, rk, fit, basis: constant velocity, shared operators against the per-element
     # solve (reached through an element map whose node counts are all equal)
     (6, 5, 9, (1.0, 0.5), 0, 3, 4, 0, 0),
-    (5, 4, 2, (-1.0, 0.5), 1, 7, 4, 0, 0),
+    (5, 4, 2, (-1.0, 0.5), 1, 3, 4, 0, 0),       # (n = 2: the faces fix every value, no energy row)
     (5, 4, 5, (0.6, -0.9), 1, 7, 3, 0, 1),
     (5, 4, 6, (0.6, -0.9), 1, 2, 2, 0, 0),
     (5, 4, 6, (-0.6, -0.9), 1, 4, 1, 0, 0),
