@@ -155,7 +155,8 @@ typedef struct {
   int fit;               /* SL_FIT_HARD or SL_FIT_SOFT                                      */
   int bvalue;            /* SL_BV_INTERP or SL_BV_BACKTRACK                                 */
   double picard_rtol;    /* energy iteration stops when max|change| < rtol * max|phihat|;
-                            0 selects 1e-13                                                 */
+                            0 selects 1e-13 (2D FP64: where phihat is zero throughout, the
+                            tolerance is never met and the linear fit is kept)              */
   int picard_cap;        /* iteration cap, 0 selects 60                                     */
 } sl_options;
 

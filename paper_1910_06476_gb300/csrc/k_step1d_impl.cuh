@@ -318,13 +318,17 @@ __device__ __forceinline__ void load_tables(const StepParams& P, const Tables1D&
   }
 }
 
-// Phase 2 of element e (eraw before the periodic wrap): phi its values, ph its remap; uface(side, c): the
-// velocity at a face at t + c dt
+// whether a double is finite, from its high word (an integer test)
+__device__ __forceinline__ bool finite64(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
+
+// Phase 2 of element e (eraw before the periodic wrap): phi its values, ph its remap, dm the mass of phi less
+// that of ph (read by the hard fit with the mass row); uface(side, c): the velocity at a face at t + c dt
 template <int NN, typename UF>
 __device__ __forceinline__ void phase2(const StepParams& P, const Smem1D& sm, int e, int eraw, const double (&phi)[NN],
-                                       const double (&ph)[NN], UF uface, double* __restrict__ out, unsigned* status) {
+                                       const double (&ph)[NN], double dm, UF uface, double* __restrict__ out,
+                                       unsigned* status) {
   const int tid = threadIdx.x, K = P.K;
-  const double h = P.hx;
+  const double lam = P.lam;              // dt / h
   const bool perW = P.bc[0] == SL_BC_PERIODIC, perE = P.bc[1] == SL_BC_PERIODIC;
   const bool bnd = (P.cons & SL_C_BOUNDARY) != 0, mass = (P.cons & SL_C_MASS) != 0;
   double d[3] = {0.0, 0.0, 0.0};        // right-hand sides of the rows left, right, mass
@@ -367,12 +371,6 @@ __device__ __forceinline__ void phase2(const StepParams& P, const Smem1D& sm, in
       }
     }
   }
-  if (mass) {
-    double Mn = 0.0;
-#pragma unroll
-    for (int i = 0; i < NN; ++i) Mn += sm.w[i] * phi[i];
-    d[2] = Mn - P.dt / h * netm;        // reference-measure target (eq. remap_mass)
-  }
   // linear constrained fit; rows are skipped where their residual vanishes (an outflow face's own trace)
   double phL[NN];
   if (P.fit == SL_FIT_HARD) {
@@ -388,12 +386,7 @@ __device__ __forceinline__ void phase2(const StepParams& P, const Smem1D& sm, in
       r0 = d[0] - c0;
       r1 = d[1] - c1;
     }
-    if (mass) {
-      double cm = 0.0;
-#pragma unroll
-      for (int j = 0; j < NN; ++j) cm += sm.w[j] * ph[j];
-      r2 = d[2] - cm;
-    }
+    if (mass) r2 = dm - lam * netm;       // reference-measure target (eq. remap_mass) less the mass of ph
 #pragma unroll
     for (int j = 0; j < NN; ++j) phL[j] = ph[j];
     if (r0 != 0.0) {
@@ -409,6 +402,12 @@ __device__ __forceinline__ void phase2(const StepParams& P, const Smem1D& sm, in
       for (int j = 0; j < NN; ++j) phL[j] += sm.Cp[2][j] * r2;
     }
   } else {
+    if (mass) {
+      double Mn = 0.0;
+#pragma unroll
+      for (int i = 0; i < NN; ++i) Mn += sm.w[i] * phi[i];
+      d[2] = Mn - lam * netm;
+    }
 #pragma unroll
     for (int j = 0; j < NN; ++j) {
       double acc = 0.0;
@@ -428,7 +427,7 @@ __device__ __forceinline__ void phase2(const StepParams& P, const Smem1D& sm, in
     double En = 0.0;
 #pragma unroll
     for (int i = 0; i < NN; ++i) En += sm.w[i] * phi[i] * phi[i];
-    const double Et = En - P.dt / h * nete;
+    const double Et = En - lam * nete;
     double EL = 0.0;
 #pragma unroll
     for (int i = 0; i < NN; ++i) EL += sm.w[i] * phL[i] * phL[i];
@@ -516,7 +515,7 @@ __device__ __forceinline__ void phase2(const StepParams& P, const Smem1D& sm, in
 #pragma unroll
   for (int i = 0; i < NN; ++i) {
     out[(size_t)e * NN + i] = res_phi[i];
-    finite = finite && isfinite(res_phi[i]);
+    finite = finite && finite64(res_phi[i]);
   }
   unsigned bits = (finite ? 0u : SL_ST_NONFINITE) | (ok ? 0u : SL_ST_PICARD_NOCONV);
   if (bits) atomicOr(status, bits);
@@ -715,7 +714,12 @@ __global__ void __launch_bounds__(BLOCK) k_step1d_f64(StepParams P, Tables1D tb,
     nodal1d<NN>(P, sm.xi, sm.lam, xk + (side ? h : 0.0), P.t + c * P.dt, u, dv);
     return u;
   };
-  phase2<NN>(P, sm, e, eraw, phi, ph, uface, out, status);
+  double dm = 0.0;
+  if ((P.cons & SL_C_MASS) && P.fit == SL_FIT_HARD) {
+#pragma unroll
+    for (int i = 0; i < NN; ++i) dm += sm.w[i] * (phi[i] - ph[i]);
+  }
+  phase2<NN>(P, sm, e, eraw, phi, ph, dm, uface, out, status);
 }
 
 // Constant velocity: phihat = R phi^n and the outflow face's values at the feet E_s phi^n, the same matrices
@@ -725,6 +729,7 @@ template <int NN>
 struct Shift1DOps {
   double R[NN * NN], E[3][NN], bs[3];
   double L[2][NN];                          // interface values: of phihat at the faces, or (eq. 4.11) of phi^n at
+  double Km[NN];                            // w - R^T w: the mass of phi^n less that of phihat
   int nst, back;                            // the faces' feet when backtracked
 };
 
@@ -781,7 +786,12 @@ __global__ void __launch_bounds__(BLOCK, NN <= 6 ? 4 : NN <= 9 ? 3 : 2) k_step1d
   }
   __syncthreads();
   if (!core) return;
-  phase2<NN>(P, sm, e, eraw, phi, ph, [&](int, double) { return a; }, out, status);
+  double dm = 0.0;
+  if (P.cons & SL_C_MASS) {
+#pragma unroll
+    for (int i = 0; i < NN; ++i) dm = fma(O.Km[i], phi[i], dm);
+  }
+  phase2<NN>(P, sm, e, eraw, phi, ph, dm, [&](int, double) { return a; }, out, status);
 }
 
 // Threads per CTA: the size whose CTAs leave the busiest SM the fewest warps (a short mesh is spread over
@@ -810,6 +820,7 @@ void launch_n(const StepParams& p, const Tables1D& tb, const Shift1D* h, const d
       std::copy(h->E[k], h->E[k] + NN, O.E[k]);
       O.bs[k] = h->bs[k];
     }
+    std::copy(h->Km, h->Km + NN, O.Km);
     O.nst = h->nst;
     O.back = p.bvalue == SL_BV_BACKTRACK;
     for (int k = 0; k < 2; ++k) std::copy(O.back ? h->B[k] : h->L[k], (O.back ? h->B[k] : h->L[k]) + NN, O.L[k]);

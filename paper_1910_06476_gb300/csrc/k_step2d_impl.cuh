@@ -929,6 +929,7 @@ __global__ void __launch_bounds__(Shape<NN>::NTMAX, Shape<NN>::MINB2)
     for (int f = 0; f < 4; ++f) SL[tid].rows[f] = 0;
     SL[tid].on = SL[tid].G.valid;
     SL[tid].mx = 0;
+    SL[tid].feasible = 0;
   }
   __syncthreads();
   const int slot = tid / ND < slots ? tid / ND : 0;
@@ -1045,9 +1046,20 @@ __global__ void __launch_bounds__(Shape<NN>::NTMAX, Shape<NN>::MINB2)
       // Equal in every thread of a slot:
       bool on = part && S.on, conv = false;
       const bool apply = on;
-      if (on) atomicMax(&S.mx, hi_abs(ph));
+      if (on) {
+        atomicMax(&S.mx, hi_abs(ph));
+        if (ph != 0.0) S.feasible = 1;
+      }
       __syncthreads();
-      if (tid < slots) SL[tid].ht = hi_abs(P.picard_rtol * fmax(hi_value(SL[tid].mx), 1e-300));
+      // where phihat vanishes identically the tolerance is zero and no change is below it: the linear fit
+      // stays, without the sixty iterations that find that out
+      if (tid < slots) {
+        Slot2<NN>& T = SL[tid];
+        T.ht = hi_abs(P.picard_rtol * fmax(hi_value(T.mx), 1e-300));
+        T.on = T.on && T.feasible;
+      }
+      __syncthreads();
+      on = on && S.on;
       for (int it = 0; it < P.picard_cap; ++it) {
         double a = 0.0, q = 0.0;
         if (on) {
@@ -1136,7 +1148,7 @@ __global__ void __launch_bounds__(Shape<NN>::NTMAX, Shape<NN>::MINB2)
   }
   if (part) {
     out[S.G.base + nd] = cur;
-    if (!isfinite(cur)) atomicOr(status, SL_ST_NONFINITE);
+    if (hi_abs(cur) >= 0x7ff00000) atomicOr(status, SL_ST_NONFINITE);
     if (!ok && nd == 0) atomicOr(status, SL_ST_PICARD_NOCONV);
   }
 }

@@ -35,6 +35,11 @@ void build_shift1d(const Basis1D& B, double a, double dt, double h, int rk, Shif
     S.bs[s] = s < S.nst ? ds_b[rk][s] : 0.0;
     basis_row(B, a > 0.0 ? 1.0 : 0.0, s < S.nst ? -ds_c[rk][s] * sx : 0.0, S.E[s]);
   }
+  for (int i = 0; i < B.n; ++i) {
+    double m = B.w[i];
+    for (int j = 0; j < B.n; ++j) m -= B.w[j] * S.R[j * B.n + i];
+    S.Km[i] = m;
+  }
   for (int f = 0; f < 2; ++f) {
     const std::vector<double>& l = f ? B.l1 : B.l0;
     std::copy(l.begin(), l.end(), S.L[f]);

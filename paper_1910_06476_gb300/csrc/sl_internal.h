@@ -99,6 +99,7 @@ struct Shift1D {
   int rk = 0, nst = 0;
   double R[NMAX * NMAX], E[3][NMAX], bs[3];
   double L[2][NMAX], B[2][NMAX];             // basis at the faces, and at their backward feet from t^{n+1}
+  double Km[NMAX];                           // w - R^T w
 };
 void build_shift1d(const Basis1D& B, double a, double dt, double h, int rk, Shift1D& S);
 // h: operators of a constant velocity, else null; xi_host: the nodes
