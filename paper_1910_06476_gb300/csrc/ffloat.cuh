@@ -51,4 +51,46 @@ struct cdot {
   __device__ __forceinline__ ff get() const { return fast_two_sum(s, c); }
 };
 
+// ------------------------------------------------------------------ two values at once
+// The same operations on one value per lane of the paired FP32 instructions, rounded like the scalar forms
+// (a - b is formed as fma(b, -1, a), the same single rounding).
+struct ff2 {
+  float2 hi, lo;
+};
+__device__ __forceinline__ float2 dup(float a) { return make_float2(a, a); }
+__device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, dup(-1.0f), a); }
+__device__ __forceinline__ ff2 two_sum2(float2 a, float2 b) {
+  const float2 s = __fadd2_rn(a, b), bb = sub2(s, a);
+  return {s, __fadd2_rn(sub2(a, sub2(s, bb)), sub2(b, bb))};
+}
+__device__ __forceinline__ ff2 fast_two_sum2(float2 a, float2 b) {
+  const float2 s = __fadd2_rn(a, b);
+  return {s, sub2(b, sub2(s, a))};
+}
+__device__ __forceinline__ ff2 ff_add2(ff2 a, ff2 b) {
+  const ff2 s = two_sum2(a.hi, b.hi);
+  return fast_two_sum2(s.hi, __fadd2_rn(__fadd2_rn(a.lo, b.lo), s.lo));
+}
+__device__ __forceinline__ ff2 ff_mul2(ff2 a, float2 wh, float2 wl) {
+  const float2 p = __fmul2_rn(a.hi, wh);
+  const float2 e = __ffma2_rn(a.hi, wh, neg2(p));
+  return fast_two_sum2(p, __ffma2_rn(a.hi, wl, __ffma2_rn(a.lo, wh, e)));
+}
+// Minus the compensated dot product of cdot, one per lane: accumulating -w v keeps every step one paired
+// instruction (a negated operand would cost two integer instructions per term)
+struct cdot2n {
+  float2 s = {0.0f, 0.0f}, c = {0.0f, 0.0f};
+  // nwh = -wh
+  __device__ __forceinline__ void add(float2 wh, float2 nwh, float2 wl, float2 hi, float2 lo) {
+    const float2 np = __fmul2_rn(nwh, hi);                        // -fl(wh hi)
+    float2 e = __ffma2_rn(wh, hi, np);                            // wh hi - fl(wh hi), exact
+    e = __ffma2_rn(wl, hi, __ffma2_rn(wh, lo, e));
+    const ff2 t = two_sum2(s, np);
+    s = t.hi;
+    c = sub2(__fadd2_rn(c, t.lo), e);
+  }
+  __device__ __forceinline__ ff2 get() const { return fast_two_sum2(s, c); }
+};
+
 }  // namespace sl

@@ -142,7 +142,13 @@ bool build_mixed1d(const sl_ctx* c, const FitOps& fit, double a, double dt, unsi
       P.Gp[pr][i] = make_float2(P.Gs[2 * pr * n + i], P.Gs[(2 * pr + 1) * n + i]);
       P.Gp[pr][n + i] = make_float2(P.Gu[2 * pr * n + i], P.Gu[(2 * pr + 1) * n + i]);
     }
-  for (int j = 0; j < n; ++j) P.w[j] = (float)w[j];
+  for (int j = 0; j < n; ++j) {
+    P.w[j] = (float)w[j];
+    P.rout[j] = (float)rout[j];
+    auto entry = [&](int k) { return fitmode == SL_FIT_HARD ? (ld)fit.Cpinv[j * m + k] : (ld)fit.SCt[j * m + k]; };
+    P.ui[j] = cons & SL_C_BOUNDARY ? (float)entry(left_up ? 0 : 1) : 0.0f;
+    P.um[j] = cons & SL_C_MASS ? (float)(lam * entry(m - 1)) : 0.0f;
+  }
   for (int s = 0; s < P.nst; ++s) {
     P.fb[s] = (float)fb[s];
     for (int j = 0; j < n; ++j) P.E[s][j] = (float)feet[s][j];

@@ -253,6 +253,9 @@ struct Mixed1DParams {
   int refine;
   float lam_lo, sumf;
   float Ff[NMAX], wh[NMAX], wl[NMAX], cmass[NMAX];
+  // Gu = ui rout^T + um f^T: the upwind element's outflow trace and outflow flux functionals (relative to its
+  // reference) and the columns they enter by (zero without their row)
+  float rout[NMAX], ui[NMAX], um[NMAX];
 };
 
 bool build_mixed1d(const sl_ctx* c, const FitOps& fit, double a, double dt, unsigned cons, int rk, int fitmode,
