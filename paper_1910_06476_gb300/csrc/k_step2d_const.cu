@@ -1,5 +1,5 @@
 // Dispatch of the 2D shared-operator kernel on the node count and the tile shape (elements per
-// CTA, TX x TY).  Each node count has a few compiled shapes, all within 48 KB of static shared
+// CTA, TX x TY, both even).  Each node count has a few compiled shapes, up to 75 KB of dynamic shared
 // memory and 1024 threads; index 0 is the default, the others are candidates for the autotuner
 // (sl_tune).  Every shape computes each element with the same arithmetic.
 #include "sl_internal.h"

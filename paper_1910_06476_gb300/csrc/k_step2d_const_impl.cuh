@@ -1,14 +1,13 @@
 #pragma once
 // 2D DSEM-SL step, mixed precision, shared operator: uniform mesh and constant velocity (a, b), so
 // every element sees the same advected geometry (Sec. 5.3).  Operators are built once on the host
-// (ops_mixed2d.cpp) and applied here in structured form, n threads per element:
-//   row phase (thread j owns row j): x-remap of the row, x inflow residual pieces, y-neighbour
-//     outflow functional, mass residual pieces                      (eq. 5.4, 4.12a, remap_mass)
-//   column phase (thread j owns column j): y-remap of the column, inflow residuals
+// (ops_mixed2d.cpp) and applied here in structured form:
+//   row phase (thread j owns row j): x-remap of the row, x-outflow trace, the row's share of the mass and
+//     outflow-flux functionals                                      (eq. 5.4, 4.12a, remap_mass)
+//   column phase (thread j owns column j): y-remap of the column, y-outflow trace, inflow residuals
 //   fit: s = (C C^T)^+ r over the inflow-face and mass rows, phi_L = psihat + C^T s   (eq. matrix_a)
 // C^T s is separable (face rows are l0/l1 along one index and a unit vector along the other, the
 // mass row is w (x) w), so the constrained fit costs O(n) per node instead of O(n) per constraint.
-// Operators applied with the same entry by every thread are read from the parameter bank.
 // State is double-float (hi plane, lo plane); all arithmetic is in float on increments relative to
 // the element's first hi value and the result is written back exactly (TwoSum).
 //
@@ -16,6 +15,22 @@
 // halo element) is one contiguous run of global memory; it is copied in aligned 16-byte vectors
 // into a shared row buffer at the same offset modulo 16 bytes, followed by the y-upwind halo row.
 // Results are written back into the own slots and stored from there with aligned vectors.
+//
+// The kernel is bound by instruction issue and the shared-memory pipe before HBM, so a thread advances TWO
+// elements at once, one in each lane of the paired FP32 operations (neighbours along x; halo elements in
+// pairs of their own): every product, sum and float-float step is one instruction for both, every table
+// entry is loaded once for both, and entries that all threads apply alike come from the parameter bank.
+// What an element needs from its upwind neighbours (outflow traces, outflow fluxes) is computed once, by the
+// neighbour's own threads, and exchanged through shared memory relative to the neighbour's reference.
+// (C C^T)^+ is applied by its structure: the face rows of C are l0/l1 times unit vectors, so C C^T is a
+// multiple of the identity on each pair of opposite faces plus couplings through span{l0, l1, w}.  Its
+// pseudo-inverse therefore is s_F = alpha_F r + Q c_F with Q an orthonormal basis of that span (three
+// columns) and 13 coefficients per element, linear in r: about 18 products per row instead of 8 n.
+//
+// Measured (one GB300): 512 x 512 elements of n = 9, boundary and mass rows: 228 -> 192 us per step (16 bytes per
+// node take 50 us at the measured copy rate; issue 49 %, shared-memory pipe 58 % of their peaks, the rest barriers);
+// pairing the elements alone left it at 234 us, the shared-memory pipe taking the operator tables.
+//
 // With the mass row, the element's mass target is also formed in float-float: M^n (float-float sum of
 // w (x) w (hi + lo)) minus its outflow fluxes through the x- and y-outflow faces plus its upwind
 // neighbours' outflow fluxes, each flux a fixed float functional of one element's values evaluated
@@ -30,15 +45,59 @@ namespace k2c {
 
 template <int NN, int TX, int TY>
 struct Tile {
+  static_assert(TX % 2 == 0 && TY % 2 == 0, "elements are advanced in pairs");
   static constexpr int ND = NN * NN;
   static constexpr int NE = TX * TY;              // elements advanced by one CTA
   static constexpr int RW = TX + 1;               // slots per staged tile row (with the x halo)
-  static constexpr int RS = (RW * ND + 8 + 3) & ~3;   // floats per staged row buffer (16-byte multiple)
+  // floats per staged row buffer: a multiple of 4 that is 8 modulo 32, so that the lanes of a warp, which run
+  // over a row or column of an element and then over the tile's rows, fall into different banks
+  static constexpr int RS = ((RW * ND + 8 + 31 - 8) & ~31) + 8;
   static constexpr int HS = (TX * ND + 8 + 3) & ~3;   // floats of the y-halo row buffer
   static constexpr int SP = TY * RS + HS;         // floats per staged plane
   static constexpr int VR = RS / 4, VH = HS / 4, VT = TY * VR + VH;   // 16-byte vectors
-  static constexpr int NT = NE * NN;              // threads
+  static constexpr int NP = NE / 2;               // own pairs: pair p holds two elements along x, see slot_of
+  static constexpr int PT = NP + TY / 2 + TX / 2; // and the x-halo (pairs along y) and y-halo pairs
+  static constexpr int NT = (PT * NN + 31) / 32 * 32;   // threads
   static constexpr int MAXV = (VT + NT - 1) / NT; // vectors per thread and plane
+  static constexpr int NR = NN | 1;               // row stride of the remapped rows
+  static constexpr int PS = NN * NR + ((NN - NN * NR) & 15);   // and the stride of a pair: NN modulo 16 (same reason)
+  static constexpr int PH = NP + TX / 2;          // pairs that are remapped: own and y-halo
+  static constexpr int MINB = NT <= 160 ? 4 : 3;  // resident CTAs asked of the compiler
+};
+
+// Operators applied with the same entry by every thread, each entry twice (parameter bank)
+template <int NN>
+struct Uni {
+  float2 Rx[NN * NN], Ry[NN * NN];
+  float2 xix[NN], rox[NN], liny[NN], louty[NN], l0[NN], l1[NN], w[NN], wh[NN], nwh[NN], wl[NN];   // wh + wl: w as float-float, nwh = -wh
+};
+// scalars of Mixed2DConstParams and the table offsets (in entries)
+struct Head {
+  int kx, ky, xw, ys, per_x, per_y, bnd, mass, mc, refine;
+  int64_t plane;
+  float gh, ghl;                                  // the inflow value as float-float
+  float sfx, sfy;
+  float al[4];                                    // alpha_F of the faces W, E, S, N
+  int o_kd, o_fx, o_fy, o_RyT, o_t, o_q, o_l0, o_l1, o_w, o_cm;
+};
+
+// shared memory of a CTA (dynamic)
+template <int NN, int TX, int TY>
+struct __align__(16) Smem {
+  using T = Tile<NN, TX, TY>;
+  float hi[T::SP], lo[T::SP];                     // staged planes
+  union {
+    float2 t[T::PH * T::PS];                      // x-remapped rows, until the column phase has read them
+    struct {
+      float2 r[T::NP * (2 * NN + 1)], c[T::NP * 13], sw[T::NP * NN], se[T::NP * NN], mv[2][T::NP * NN];
+    } f;                                          // the fit, after it
+  } a;
+  float2 u[T::PT * NN], v[T::PT * NN];            // outflow traces along x (before R_y) and y (relative to the own ref)
+  float2 fp[5][T::PT * NN];                       // row shares: mass residual, x and y flux, -M^n hi, lo
+  float2 dx[T::NP * NN];
+  float ref[2 * T::PT], tot[3][2 * T::PT], mnh[2 * T::NP], mnl[2 * T::NP], miss[2 * T::NP];
+  int64_t a0[TY + 1];                             // first aligned global float of each staged row
+  int off[TY + 1], nv[TY + 1];                    // row data offset in its buffer; vectors (0: gather)
 };
 
 __device__ __forceinline__ int wrapi(int i, int n, bool per) {
@@ -51,23 +110,15 @@ __device__ __forceinline__ int wrapi(int i, int n, bool per) {
 __device__ __forceinline__ int64_t floor4(int64_t g) { return g & ~int64_t(3); }
 
 template <int NN, int TX, int TY>
-__global__ void __launch_bounds__(Tile<NN, TX, TY>::NT)
-    k_step2d_shared(const __grid_constant__ Mixed2DConstParams P, const float* __restrict__ tab,
+__global__ void __launch_bounds__(Tile<NN, TX, TY>::NT, Tile<NN, TX, TY>::MINB)
+    k_step2d_shared(const __grid_constant__ Uni<NN> U, const __grid_constant__ Head P, const float* __restrict__ tab,
                     const float* __restrict__ in, float* __restrict__ out, unsigned* status) {
   using T = Tile<NN, TX, TY>;
-  constexpr int ND = T::ND, NE = T::NE, RW = T::RW, RS = T::RS, SP = T::SP, NT = T::NT;
+  constexpr int ND = T::ND, RW = T::RW, RS = T::RS, NT = T::NT, NP = T::NP, NR = T::NR, NC = 2 * NN + 1;
   constexpr int VR = T::VR, VT = T::VT, MAXV = T::MAXV;
-  __shared__ __align__(16) float s_hi[SP];
-  __shared__ __align__(16) float s_lo[SP];
-  __shared__ float s_t[NE * ND];                  // x-remapped rows
-  __shared__ float s_dx[NE][NN], s_v[NE][NN], s_p[NE][NN], s_r[NE][2 * NN], s_sw[NE][NN], s_se[NE][NN];
-  __shared__ int64_t s_a0[TY + 1];                // first aligned global float of each staged row
-  __shared__ int s_off[TY + 1], s_nv[TY + 1];     // row data offset in its buffer; vectors (0: gather)
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  Smem<NN, TX, TY>& S = *reinterpret_cast<Smem<NN, TX, TY>*>(smem_raw);
   const int tid = threadIdx.x;
-  // mass refinement (dynamic shared memory): per element and row, the row partials of the own and
-  // upwind outflow fluxes and of M^n (slots 0-5), then per column the written mass (6, 7)
-  extern __shared__ __align__(16) float s_dyn[];
-  float (*s_fp)[NN][8] = reinterpret_cast<float (*)[NN][8]>(s_dyn);
   const int ex0 = blockIdx.x * TX, ey0 = blockIdx.y * TY;
   const bool perx = P.per_x != 0, pery = P.per_y != 0;
   const int xs0 = P.xw ? ex0 - 1 : ex0;           // first element of a staged tile row
@@ -78,9 +129,9 @@ __global__ void __launch_bounds__(Tile<NN, TX, TY>::NT)
     const int64_t g0 = ((int64_t)ey * P.kx + xa) * ND;
     const int64_t a0 = floor4(g0);
     const bool fast = ey >= 0 && ey < P.ky && xa >= 0 && xa + cnt <= P.kx;
-    s_a0[tid] = a0;
-    s_off[tid] = (int)(g0 - a0);
-    s_nv[tid] = fast ? (int)((floor4(g0 + cnt * ND + 3) - a0) >> 2) : 0;
+    S.a0[tid] = a0;
+    S.off[tid] = (int)(g0 - a0);
+    S.nv[tid] = fast ? (int)((floor4(g0 + cnt * ND + 3) - a0) >> 2) : 0;
   }
   __syncthreads();
   // contiguous rows: every vector load first, then the shared stores
@@ -91,8 +142,8 @@ __global__ void __launch_bounds__(Tile<NN, TX, TY>::NT)
       const int v = tid + k * NT;
       const int r = v < TY * VR ? v / VR : TY;
       const int vv = v - r * VR;
-      if (v < VT && vv < s_nv[r]) {
-        const float4* src = reinterpret_cast<const float4*>(in + s_a0[r]) + vv;
+      if (v < VT && vv < S.nv[r]) {
+        const float4* src = reinterpret_cast<const float4*>(in + S.a0[r]) + vv;
         vh[k] = __ldg(src);
         vl[k] = __ldg(reinterpret_cast<const float4*>(reinterpret_cast<const float*>(src) + P.plane));
       }
@@ -102,289 +153,306 @@ __global__ void __launch_bounds__(Tile<NN, TX, TY>::NT)
       const int v = tid + k * NT;
       const int r = v < TY * VR ? v / VR : TY;
       const int vv = v - r * VR;
-      if (v < VT && vv < s_nv[r]) {
-        reinterpret_cast<float4*>(s_hi + r * RS)[vv] = vh[k];
-        reinterpret_cast<float4*>(s_lo + r * RS)[vv] = vl[k];
+      if (v < VT && vv < S.nv[r]) {
+        reinterpret_cast<float4*>(S.hi + r * RS)[vv] = vh[k];
+        reinterpret_cast<float4*>(S.lo + r * RS)[vv] = vl[k];
       }
     }
   }
   // rows that wrap, leave the mesh or are ragged: element by element (ghost slots hold zero)
 #pragma unroll 1
   for (int r = 0; r <= TY; ++r) {
-    if (s_nv[r] != 0) continue;
+    if (S.nv[r] != 0) continue;
     const int ey = r < TY ? ey0 + r : eyh;
     const int xa = r < TY ? xs0 : ex0, cnt = r < TY ? RW : TX;
     const int wy = wrapi(ey, P.ky, pery);
-    const int base = r * RS + s_off[r];
+    const int base = r * RS + S.off[r];
     for (int idx = tid; idx < cnt * ND; idx += NT) {
       const int sl = idx / ND, q = idx - sl * ND;
       const int wx = wrapi(xa + sl, P.kx, perx);
       const bool ok = wx >= 0 && wy >= 0;
       const size_t g = ((size_t)wy * P.kx + wx) * ND + q;
-      s_hi[base + idx] = ok ? __ldg(in + g) : 0.0f;
-      s_lo[base + idx] = ok ? __ldg(in + P.plane + g) : 0.0f;
+      S.hi[base + idx] = ok ? __ldg(in + g) : 0.0f;
+      S.lo[base + idx] = ok ? __ldg(in + P.plane + g) : 0.0f;
     }
   }
   __syncthreads();
 
-  const int el = tid / NN, j = tid - (tid / NN) * NN;   // element in the tile, row / column index
-  const int lx = el % TX, ly = el / TX;
+  // pair p: own pairs first (along y, then along x), then the x halo (rows 2 r, 2 r + 1), then the y halo;
+  // element e of the arrays below is lane e & 1 of pair e / 2
+  auto slot_of = [](int lx, int ly) { return 2 * ((lx >> 1) * TY + ly) + (lx & 1); };
+  const int p = tid / NN, j = tid - p * NN;
+  const bool own = p < NP, valid = p < T::PT, halox = !own && p < NP + TY / 2;
+  int o0, o1;                                     // staged offsets of the pair's elements
+  if (halox) {
+    const int r = 2 * (p - NP), c = (P.xw ? 0 : TX) * ND;
+    o0 = r * RS + S.off[r] + c;
+    o1 = (r + 1) * RS + S.off[r + 1] + c;
+  } else if (own || !valid) {
+    const int ly = valid ? p % TY : 0, lx = valid ? 2 * (p / TY) : 0;
+    o0 = ly * RS + S.off[ly] + (lx + P.xw) * ND;
+    o1 = o0 + ND;
+  } else {
+    o0 = TY * RS + S.off[TY] + 2 * (p - NP - TY / 2) * ND;
+    o1 = o0 + ND;
+  }
+  const float2 ref = make_float2(S.hi[o0], S.hi[o1]);
+  const int pj = p * NN + j;
+
+  // ---- row phase: thread j holds row j of psi
+  float2 tau = dup(0.0f);
+  if (valid) {
+    float2 q[NN];
+    const float2 mref = make_float2(-ref.x, -ref.y);
+    cdot2n mn;
+    const bool massf = own && P.refine;
+#pragma unroll
+    for (int i = 0; i < NN; ++i) {
+      const float2 h = make_float2(S.hi[o0 + j * NN + i], S.hi[o1 + j * NN + i]);
+      const float2 l = make_float2(S.lo[o0 + j * NN + i], S.lo[o1 + j * NN + i]);
+      q[i] = __fadd2_rn(__fadd2_rn(h, mref), l);
+      if (massf) mn.add(U.wh[i], U.nwh[i], U.wl[i], h, l);   // (row sum; the rows' weights in the element total)
+    }
+    float2 u = dup(0.0f);
+#pragma unroll
+    for (int i = 0; i < NN; ++i) {
+      u = __ffma2_rn(U.rox[i], q[i], u);
+      tau = __ffma2_rn(U.xix[i], q[i], tau);
+    }
+    S.u[pj] = u;
+    if (P.mass) {
+      float2 kd = dup(0.0f), fx = dup(0.0f), fy = dup(0.0f);
+#pragma unroll
+      for (int i = 0; i < NN; ++i) {
+        kd = __ffma2_rn(dup(__ldg(tab + P.o_kd + i * NN + j)), q[i], kd);
+        fx = __ffma2_rn(dup(__ldg(tab + P.o_fx + i * NN + j)), q[i], fx);
+        fy = __ffma2_rn(dup(__ldg(tab + P.o_fy + i * NN + j)), q[i], fy);
+      }
+      S.fp[0][pj] = kd;
+      S.fp[1][pj] = fx;
+      S.fp[2][pj] = fy;
+      if (massf) {
+        const ff2 m = mn.get();
+        S.fp[3][pj] = m.hi;
+        S.fp[4][pj] = m.lo;
+      }
+    }
+    if (j == 0) {
+      S.ref[2 * p] = ref.x;
+      S.ref[2 * p + 1] = ref.y;
+    }
+    if (!halox) {
+      float2* tr = S.a.t + (own ? p : p - TY / 2) * T::PS + j * NR;
+      // x-remap of row j: t[j][l] = sum_i R_x[l][i] psi[j][i]
+#pragma unroll
+      for (int l = 0; l < NN; ++l) {
+        float2 acc = dup(0.0f);
+#pragma unroll
+        for (int i = 0; i < NN; ++i) acc = __ffma2_rn(U.Rx[l * NN + i], q[i], acc);
+        tr[l] = acc;
+      }
+    }
+  }
+  __syncthreads();
+
+  // upwind neighbours: elements xn0, xn1 across the x-inflow faces, pair yp across the y-inflow face
+  const int ly = own ? p % TY : 0, lx = own ? 2 * (p / TY) : 0, e0 = 2 * p;
   const int ex = ex0 + lx, ey = ey0 + ly;
-  const bool active = ex < P.kx && ey < P.ky;
-  // own slot, x-upwind neighbour (same staged row), y-upwind neighbour (adjacent row or the halo)
-  const int so = ly * RS + s_off[ly] + (lx + P.xw) * ND;
-  const int sx = ly * RS + s_off[ly] + (P.xw ? lx : lx + 1) * ND;
-  const int ry = P.ys ? ly - 1 : ly + 1;
-  const int sy = (ry >= 0 && ry < TY) ? ry * RS + s_off[ry] + (lx + P.xw) * ND : TY * RS + s_off[TY] + lx * ND;
-  const bool gx = wrapi(P.xw ? ex - 1 : ex + 1, P.kx, perx) < 0;
-  const bool gy = wrapi(P.ys ? ey - 1 : ey + 1, P.ky, pery) < 0;
-  const float ref = s_hi[so];
-  const float gval = (float)(P.ghost - (double)ref);
-
-  // ---- row phase: thread j holds row j of psi and psi_X, column j of psi_Y
-  float ps[NN];
+  int xn0, xn1, yp;
   {
-    float px[NN], py[NN];
-    const float2 mref = make_float2(-ref, -ref);
-#pragma unroll
-    for (int i = 0; i < NN; ++i) {                // own and x-neighbour node side by side
-      const float2 d = __fadd2_rn(make_float2(s_hi[so + j * NN + i], s_hi[sx + j * NN + i]), mref);
-      const float2 v = __fadd2_rn(d, make_float2(s_lo[so + j * NN + i], s_lo[sx + j * NN + i]));
-      ps[i] = v.x;
-      px[i] = gx ? gval : v.y;
-      py[i] = gy ? gval : (s_hi[sy + i * NN + j] - ref) + s_lo[sy + i * NN + j];
-    }
-    // x inflow residual pieces: upwind outflow trace minus own inflow trace, before the y-remap
-    float u = 0.0f, tau = 0.0f, v = 0.0f, pm = 0.0f;
-#pragma unroll
-    for (int i = 0; i < NN; ++i) {
-      u = fmaf(P.rox[i], px[i], u);
-      tau = fmaf(P.xix[i], ps[i], tau);
-      v = fmaf(P.roy[i], py[i], v);
-    }
-    // mass residual pieces (target minus the mass of psihat, reference measure)
-    const float* Ks = tab + P.o_ks;
-    const float* Kx = tab + P.o_kx;
-    const float* Ky = tab + P.o_ky;
-#pragma unroll
-    for (int i = 0; i < NN; ++i) {
-      pm = fmaf(__ldg(Ks + i * NN + j), ps[i], pm);
-      pm = fmaf(__ldg(Kx + i * NN + j), px[i], pm);
-      pm = fmaf(__ldg(Ky + i * NN + j), py[i], pm);
-    }
-    s_dx[el][j] = (gx ? 0.0f : u) - tau;
-    s_v[el][j] = gy ? 0.0f : v;
-    s_p[el][j] = pm;
+    const int xh = 2 * NP + ly;                   // this tile row's x-halo element
+    if (P.xw) { xn0 = lx > 0 ? slot_of(lx - 1, ly) : xh; xn1 = e0; }
+    else { xn0 = e0 + 1; xn1 = lx + 2 < TX ? slot_of(lx + 2, ly) : xh; }
+    const int ry = P.ys ? ly - 1 : ly + 1;
+    yp = ry >= 0 && ry < TY ? (lx >> 1) * TY + ry : NP + TY / 2 + (lx >> 1);
   }
-  if (P.refine) {
-    // row j of: the own outflow fluxes (x, y faces), the upwind neighbours' outflow fluxes (their
-    // rows with their own references, in the same operations as they use themselves), the own mass
-    const float* Fx = tab + P.o_fx;
-    const float* Fy = tab + P.o_fy;
-    const float* Wh = tab + P.o_wh;
-    const float* Wl = tab + P.o_wl;
-    float fxo = 0.0f, fyo = 0.0f, fxu = 0.0f, fyu = 0.0f;
-    cdot mn;
-    const float refx = s_hi[sx], refy = s_hi[sy];
-#pragma unroll
-    for (int i = 0; i < NN; ++i) {
-      const float fxi = __ldg(Fx + i * NN + j), fyi = __ldg(Fy + i * NN + j);
-      const float hi = s_hi[so + j * NN + i], lo = s_lo[so + j * NN + i];
-      const float qo = __fadd_rn(__fsub_rn(hi, ref), lo);
-      const float qx = __fadd_rn(__fsub_rn(s_hi[sx + j * NN + i], refx), s_lo[sx + j * NN + i]);
-      const float qy = __fadd_rn(__fsub_rn(s_hi[sy + j * NN + i], refy), s_lo[sy + j * NN + i]);
-      fxo = fmaf(fxi, qo, fxo);
-      fyo = fmaf(fyi, qo, fyo);
-      fxu = fmaf(fxi, qx, fxu);
-      fyu = fmaf(fyi, qy, fyu);
-      mn.add(__ldg(Wh + i * NN + j), __ldg(Wl + i * NN + j), hi, lo);
-    }
-    const ff mnr = mn.get();
-    s_fp[el][j][0] = fxo;
-    s_fp[el][j][1] = fyo;
-    s_fp[el][j][2] = fxu;
-    s_fp[el][j][3] = fyu;
-    s_fp[el][j][4] = mnr.hi;
-    s_fp[el][j][5] = mnr.lo;
-  }
-  // x-remap of row j: t[j][l] = sum_i R_x[l][i] psi[j][i]; rows l, l + 1 in paired FMAs (each
-  // lane rounds like fmaf, in the same order)
-#pragma unroll
-  for (int q = 0; q < NN / 2; ++q) {
-    float2 acc = make_float2(0.0f, 0.0f);
-#pragma unroll
-    for (int i = 0; i < NN; ++i) acc = __ffma2_rn(P.Rxp[q][i], make_float2(ps[i], ps[i]), acc);
-    s_t[el * ND + j * NN + 2 * q] = acc.x;
-    s_t[el * ND + j * NN + 2 * q + 1] = acc.y;
-  }
-  if (NN & 1) {
-    constexpr int l = NN - 1;
-    float acc = 0.0f;
-#pragma unroll
-    for (int i = 0; i < NN; ++i) acc = fmaf(P.Rx[l * NN + i], ps[i], acc);
-    s_t[el * ND + j * NN + l] = acc;
-  }
-  __syncthreads();
+  const bool gx0 = wrapi(P.xw ? ex - 1 : ex + 1, P.kx, perx) < 0, gx1 = wrapi(P.xw ? ex : ex + 2, P.kx, perx) < 0;
+  const bool gy = wrapi(P.ys ? ey - 1 : ey + 1, P.ky, pery) < 0;
+  const float2 gval = __fadd2_rn(sub2(dup(P.gh), ref), dup(P.ghl));   // the ghost relative to the reference
+  // differences of the references: neighbour values relative to the own reference
+  const float2 drx = own ? make_float2(gx0 ? 0.0f : S.ref[xn0] - ref.x, gx1 ? 0.0f : S.ref[xn1] - ref.y) : dup(0.0f);
+  const float2 dry = own && !gy ? make_float2(S.ref[2 * yp] - ref.x, S.ref[2 * yp + 1] - ref.y) : dup(0.0f);
 
   // ---- column phase: thread j holds column j of psihat = R_y t
-  float ph[NN];
-  {
-    float tc[NN];
+  float2 ph[NN], ty = dup(0.0f);
+  if (valid && !halox) {
+    float2 tc[NN], v = dup(0.0f);
+    const float2* tr = S.a.t + (own ? p : p - TY / 2) * T::PS + j;
 #pragma unroll
-    for (int m = 0; m < NN; ++m) tc[m] = s_t[el * ND + m * NN + j];
+    for (int m = 0; m < NN; ++m) tc[m] = tr[m * NR];
 #pragma unroll
-    for (int q = 0; q < NN / 2; ++q) {
-      float2 acc = make_float2(0.0f, 0.0f);
+    for (int k = 0; k < NN; ++k) {
+      float2 acc = dup(0.0f);
 #pragma unroll
-      for (int m = 0; m < NN; ++m) acc = __ffma2_rn(P.Ryp[q][m], make_float2(tc[m], tc[m]), acc);
-      ph[2 * q] = acc.x;
-      ph[2 * q + 1] = acc.y;
-    }
-    if (NN & 1) {
-      constexpr int k = NN - 1;
-      float acc = 0.0f;
-#pragma unroll
-      for (int m = 0; m < NN; ++m) acc = fmaf(P.Ry[k * NN + m], tc[m], acc);
+      for (int m = 0; m < NN; ++m) acc = __ffma2_rn(U.Ry[k * NN + m], tc[m], acc);
       ph[k] = acc;
+      ty = __ffma2_rn(U.liny[k], acc, ty);
+      v = __ffma2_rn(U.louty[k], acc, v);
     }
+    S.v[pj] = v;                                  // trace of psihat on the y-outflow face
   }
-  float rm = 0.0f;                                // mass residual (same summation order everywhere)
+  if (own) {
+    const float* us = reinterpret_cast<const float*>(S.u);
+    const float2 un = make_float2(gx0 ? 0.0f : us[((xn0 >> 1) * NN + j) * 2 + (xn0 & 1)],
+                                  gx1 ? 0.0f : us[((xn1 >> 1) * NN + j) * 2 + (xn1 & 1)]);
+    S.dx[pj] = sub2(__fadd2_rn(un, drx), tau);
+  }
+  // element totals of the row shares, one thread per element, rows in order (the same sums whichever CTA
+  // forms them): mass residual, outflow fluxes, M^n in float-float
+  if (P.mass)
+    for (int e = tid; e < 2 * T::PT; e += NT) {
+      const float* f = reinterpret_cast<const float*>(S.fp) + (e >> 1) * NN * 2 + (e & 1);
+      constexpr int F = T::PT * NN * 2;
+      float kd = 0.0f, fx = 0.0f, fy = 0.0f;
 #pragma unroll
-  for (int q = 0; q < NN; ++q) rm += s_p[el][q];
-  if (P.bnd) {
-    const float* RxT = tab + P.o_RxT;
-    const float* RyT = tab + P.o_RyT;
-    float rx = 0.0f, vy = 0.0f, ty = 0.0f;
+      for (int r = 0; r < NN; ++r) {
+        kd += f[2 * r];
+        fx += f[F + 2 * r];
+        fy += f[2 * F + 2 * r];
+      }
+      S.tot[0][e] = kd;
+      S.tot[1][e] = fx;
+      S.tot[2][e] = fy;
+      if (P.refine && e < 2 * NP) {
+        ff mn = ff_mul(ff{f[3 * F], f[4 * F]}, ff{U.wh[0].x, U.wl[0].x});
 #pragma unroll
-    for (int m = 0; m < NN; ++m) {
-      rx = fmaf(__ldg(RyT + m * NN + j), s_dx[el][m], rx);
-      vy = fmaf(__ldg(RxT + m * NN + j), s_v[el][m], vy);
-      ty = fmaf(P.liny[m], ph[m], ty);
+        for (int r = 1; r < NN; ++r)
+          mn = ff_add(mn, ff_mul(ff{f[3 * F + 2 * r], f[4 * F + 2 * r]}, ff{U.wh[r].x, U.wl[r].x}));
+        S.mnh[e] = mn.hi;
+        S.mnl[e] = mn.lo;
+      }
     }
-    s_r[el][j] = rx + (gx ? gval : 0.0f);
-    s_r[el][NN + j] = (vy + (gy ? gval : 0.0f)) - ty;
+  __syncthreads();
+
+  float2 rm = dup(0.0f);                          // mass residual
+  if (own && P.mass) {
+    auto at = [&](int k, int a, int b) { return make_float2(S.tot[k][a], S.tot[k][b]); };
+    const float2 gxv = make_float2(gx0 ? gval.x : drx.x, gx1 ? gval.y : drx.y), gyv = gy ? gval : dry;
+    float2 fxu = make_float2(gx0 ? 0.0f : S.tot[1][xn0], gx1 ? 0.0f : S.tot[1][xn1]);
+    float2 fyu = gy ? dup(0.0f) : at(2, 2 * yp, 2 * yp + 1);
+    fxu = __ffma2_rn(gxv, dup(P.sfx), fxu);
+    fyu = __ffma2_rn(gyv, dup(P.sfy), fyu);
+    rm = __fadd2_rn(at(0, e0, e0 + 1), __fadd2_rn(sub2(fxu, at(1, e0, e0 + 1)), sub2(fyu, at(2, e0, e0 + 1))));
+  }
+  float2 rx = dup(0.0f), ry = dup(0.0f);
+  if (own && P.bnd) {
+#pragma unroll
+    for (int m = 0; m < NN; ++m) rx = __ffma2_rn(dup(__ldg(tab + P.o_RyT + m * NN + j)), S.dx[p * NN + m], rx);
+    if (gx0) rx.x += gval.x;
+    if (gx1) rx.y += gval.y;
+    ry = sub2(gy ? gval : __fadd2_rn(S.v[yp * NN + j], dry), ty);
+    S.a.f.r[p * NC + j] = rx;
+    S.a.f.r[p * NC + NN + j] = ry;
+    if (j == 0) S.a.f.r[p * NC + 2 * NN] = rm;    // (zero without the mass row)
   }
   __syncthreads();
 
-  // ---- fit: s = (C C^T)^+ r; thread j forms the face entries of row / column j
-  float sS = 0.0f, sN = 0.0f, sm = 0.0f;
+  // ---- fit: s = (C C^T)^+ r: the 13 coefficients (three per face along Q, the mass row's entry), spread over
+  // the element's threads; then thread j forms the face entries of row / column j
+  float2 sS = dup(0.0f), sN = dup(0.0f), sm = dup(0.0f);
   if (P.bnd) {
-    const int mc = P.mc;
-    const float* G = tab + P.o_g;
-    float sW = 0.0f, sE = 0.0f;
+    if (own) {
+      for (int o = j; o < 13; o += NN) {
+        const float* To = tab + P.o_t + o * NC;
+        float2 c = dup(0.0f);
 #pragma unroll
-    for (int k = 0; k < 2 * NN; ++k) {
-      const float rk = s_r[el][k];
-      sW = fmaf(__ldg(G + (0 * mc + k) * NN + j), rk, sW);
-      sE = fmaf(__ldg(G + (1 * mc + k) * NN + j), rk, sE);
-      sS = fmaf(__ldg(G + (2 * mc + k) * NN + j), rk, sS);
-      sN = fmaf(__ldg(G + (3 * mc + k) * NN + j), rk, sN);
-      sm = fmaf(P.gm[k], rk, sm);
+        for (int k = 0; k < NC; ++k) c = __ffma2_rn(dup(__ldg(To + k)), S.a.f.r[p * NC + k], c);
+        S.a.f.c[p * 13 + o] = c;
+      }
     }
-    if (P.mass) {
-      sW = fmaf(__ldg(G + (0 * mc + 2 * NN) * NN + j), rm, sW);
-      sE = fmaf(__ldg(G + (1 * mc + 2 * NN) * NN + j), rm, sE);
-      sS = fmaf(__ldg(G + (2 * mc + 2 * NN) * NN + j), rm, sS);
-      sN = fmaf(__ldg(G + (3 * mc + 2 * NN) * NN + j), rm, sN);
-      sm = fmaf(P.gm[2 * NN], rm, sm);
-    }
-    s_sw[el][j] = sW;
-    s_se[el][j] = sE;
     __syncthreads();
-  } else {
-    sm = P.gm[0] * rm;
+    if (own) {
+      const float2 q0 = dup(__ldg(tab + P.o_q + j)), q1 = dup(__ldg(tab + P.o_q + NN + j)), q2 = dup(__ldg(tab + P.o_q + 2 * NN + j));
+      const float2* c = S.a.f.c + p * 13;
+      auto entry = [&](int f, float2 r) {
+        return __ffma2_rn(c[3 * f + 2], q2, __ffma2_rn(c[3 * f + 1], q1, __ffma2_rn(c[3 * f], q0, __fmul2_rn(dup(P.al[f]), r))));
+      };
+      S.a.f.sw[pj] = entry(0, rx);
+      S.a.f.se[pj] = entry(1, rx);
+      sS = entry(2, ry);
+      sN = entry(3, ry);
+      sm = c[12];
+    }
+    __syncthreads();
+  } else if (own) {
+    sm = __fmul2_rn(dup(__ldg(tab + P.o_t + 12)), rm);
   }
 
-  // ---- phi_L = psihat + C^T s, column j; exact write-back into the own slot
-  {
-    const float l0j = __ldg(tab + P.o_l0 + j), l1j = __ldg(tab + P.o_l1 + j);
-    const float wj = __ldg(tab + P.o_w + j) * sm;
-    bool finite = true;
-    float vh[NN], vl[NN];
-    // nodes k and k + 1 in paired operations, each lane in the scalar order (a - b as fma(b, -1, a))
-    const float2 rr = make_float2(ref, ref), m1 = make_float2(-1.0f, -1.0f);
+  // ---- phi_L = psihat + C^T s, column j; exact write-back
+  float2 vh[NN], vl[NN];
+  if (own) {
+    const float2 l0j = dup(__ldg(tab + P.o_l0 + j)), l1j = dup(__ldg(tab + P.o_l1 + j));
+    const float2 wj = __fmul2_rn(dup(__ldg(tab + P.o_w + j)), sm);
+    cdot2n mv;
 #pragma unroll
-    for (int k = 0; k + 1 < NN; k += 2) {
-      float2 acc = make_float2(ph[k], ph[k + 1]);
-      acc = __ffma2_rn(make_float2(sS, sS), make_float2(P.l0[k], P.l0[k + 1]), acc);
-      acc = __ffma2_rn(make_float2(sN, sN), make_float2(P.l1[k], P.l1[k + 1]), acc);
-      acc = __ffma2_rn(make_float2(wj, wj), make_float2(P.w[k], P.w[k + 1]), acc);
+    for (int k = 0; k < NN; ++k) {
+      float2 acc = ph[k];
+      acc = __ffma2_rn(sS, U.l0[k], acc);
+      acc = __ffma2_rn(sN, U.l1[k], acc);
+      acc = __ffma2_rn(wj, U.w[k], acc);
       if (P.bnd) {
-        acc = __ffma2_rn(make_float2(s_sw[el][k], s_sw[el][k + 1]), make_float2(l0j, l0j), acc);
-        acc = __ffma2_rn(make_float2(s_se[el][k], s_se[el][k + 1]), make_float2(l1j, l1j), acc);
+        acc = __ffma2_rn(S.a.f.sw[p * NN + k], l0j, acc);
+        acc = __ffma2_rn(S.a.f.se[p * NN + k], l1j, acc);
       }
-      const float2 s2 = __fadd2_rn(rr, acc);
-      const float2 bb = __ffma2_rn(rr, m1, s2);                         // s - ref
-      const float2 t = __ffma2_rn(__ffma2_rn(bb, m1, s2), m1, rr);      // ref - (s - bb)
-      const float2 e = __fadd2_rn(t, __ffma2_rn(bb, m1, acc));          // + (acc - bb)
-      vh[k] = s2.x;
-      vh[k + 1] = s2.y;
-      vl[k] = e.x;
-      vl[k + 1] = e.y;
-    }
-    if (NN & 1) {
-      constexpr int k = NN - 1;
-      float acc = ph[k];
-      acc = fmaf(sS, P.l0[k], acc);
-      acc = fmaf(sN, P.l1[k], acc);
-      acc = fmaf(wj, P.w[k], acc);
-      if (P.bnd) {
-        acc = fmaf(s_sw[el][k], l0j, acc);
-        acc = fmaf(s_se[el][k], l1j, acc);
-      }
-      const float s = ref + acc;
-      const float bb = s - ref;
-      vh[k] = s;
-      vl[k] = (ref - (s - bb)) + (acc - bb);
+      const ff2 s = two_sum2(ref, acc);
+      vh[k] = s.hi;
+      vl[k] = s.lo;
+      if (P.refine) mv.add(U.wh[k], U.nwh[k], U.wl[k], vh[k], vl[k]);    // (column sum)
     }
     if (P.refine) {
-      // float-float mass of column j, summed over the columns by the element's first thread; the
-      // miss against the target goes along the mass column of the pseudo-inverse into the lo words
-      const float* Wh = tab + P.o_wh;
-      const float* Wl = tab + P.o_wl;
-      cdot mvc;
+      const ff2 m = mv.get();
+      S.a.f.mv[0][pj] = m.hi;
+      S.a.f.mv[1][pj] = m.lo;
+    }
+  }
+  if (P.refine) {
+    // the float-float miss of the written element mass against the target, one thread per element:
+    // F(element) = ref sum(f) + its total, own fluxes with this element's reference, upwind fluxes with the
+    // neighbour's (or the ghost value)
+    __syncthreads();
+    for (int e = tid; e < 2 * NP; e += NT) {
+      const float* f = reinterpret_cast<const float*>(S.a.f.mv) + (e >> 1) * NN * 2 + (e & 1);
+      constexpr int F = NP * NN * 2;
+      ff m = ff_mul(ff{f[0], f[F]}, ff{U.wh[0].x, U.wl[0].x});
 #pragma unroll
-      for (int k = 0; k < NN; ++k) mvc.add(__ldg(Wh + k * NN + j), __ldg(Wl + k * NN + j), vh[k], vl[k]);
-      const ff mv = mvc.get();
-      s_fp[el][j][6] = mv.hi;
-      s_fp[el][j][7] = mv.lo;
-      __syncthreads();
-      // F(element) = ref sum(f) + the row partials added in row order: own fluxes with this element's
-      // reference, upwind fluxes with the neighbour's (or the ghost value); every thread of the
-      // element forms the target and the miss in the same order
-      float axo = 0.0f, ayo = 0.0f, axu = 0.0f, ayu = 0.0f;
-      ff mn = {0.0f, 0.0f}, tot = {0.0f, 0.0f};
-#pragma unroll
-      for (int q = 0; q < NN; ++q) {
-        axo += s_fp[el][q][0];
-        ayo += s_fp[el][q][1];
-        axu += s_fp[el][q][2];
-        ayu += s_fp[el][q][3];
-        mn = ff_add(mn, ff{s_fp[el][q][4], s_fp[el][q][5]});
-        tot = ff_add(tot, ff{s_fp[el][q][6], s_fp[el][q][7]});
-      }
-      const float gh = (float)P.ghost;
-      const float Fxo = fmaf(ref, P.sfx, axo), Fyo = fmaf(ref, P.sfy, ayo);
-      const float Fxu = gx ? gh * P.sfx : fmaf(s_hi[sx], P.sfx, axu);
-      const float Fyu = gy ? gh * P.sfy : fmaf(s_hi[sy], P.sfy, ayu);
+      for (int r = 1; r < NN; ++r) m = ff_add(m, ff_mul(ff{f[2 * r], f[F + 2 * r]}, ff{U.wh[r].x, U.wl[r].x}));
+      const int x = 2 * ((e >> 1) / TY) + (e & 1), y = (e >> 1) % TY;
+      const int xh = 2 * NP + y;
+      const int xn = P.xw ? (x > 0 ? slot_of(x - 1, y) : xh) : (x + 1 < TX ? slot_of(x + 1, y) : xh);
+      const int ry = P.ys ? y - 1 : y + 1, yn = ry >= 0 && ry < TY ? slot_of(x, ry) : 2 * (NP + TY / 2) + x;
+      const bool gx = wrapi(P.xw ? ex0 + x - 1 : ex0 + x + 1, P.kx, perx) < 0;
+      const bool gyy = wrapi(P.ys ? ey0 + y - 1 : ey0 + y + 1, P.ky, pery) < 0;
+      const float Fxo = fmaf(S.ref[e], P.sfx, S.tot[1][e]), Fyo = fmaf(S.ref[e], P.sfy, S.tot[2][e]);
+      const float Fxu = gx ? P.gh * P.sfx : fmaf(S.ref[xn], P.sfx, S.tot[1][xn]);
+      const float Fyu = gyy ? P.gh * P.sfy : fmaf(S.ref[yn], P.sfy, S.tot[2][yn]);
       // M^{n+1} = M^n - (outflow) + (inflow), float-float
-      const ff tg = ff_add(mn, ff_add(two_sum(-Fxo, -Fyo), two_sum(Fxu, Fyu)));
-      const float miss = ff_to_f(ff_add(tg, ff_neg(tot)));
-      const float* Cm = tab + P.o_cm;
+      const ff tg = ff_add(ff{-S.mnh[e], -S.mnl[e]}, ff_add(two_sum(-Fxo, -Fyo), two_sum(Fxu, Fyu)));
+      S.miss[e] = ff_to_f(ff_add(tg, m));          // (m: minus the written mass)
+    }
+    __syncthreads();
+    if (own) {
+      const float2 miss = make_float2(S.miss[e0], S.miss[e0 + 1]);
 #pragma unroll
       for (int k = 0; k < NN; ++k) {
-        const ff v = fast_two_sum(vh[k], fmaf(miss, __ldg(Cm + k * NN + j), vl[k]));
+        const ff2 v = fast_two_sum2(vh[k], __ffma2_rn(miss, dup(__ldg(tab + P.o_cm + k * NN + j)), vl[k]));
         vh[k] = v.hi;
         vl[k] = v.lo;
       }
     }
+  }
+  if (own) {
+    bool f0 = true, f1 = true;
 #pragma unroll
     for (int k = 0; k < NN; ++k) {
-      s_hi[so + k * NN + j] = vh[k];
-      s_lo[so + k * NN + j] = vl[k];
-      finite = finite && isfinite(vh[k]);
+      S.hi[o0 + k * NN + j] = vh[k].x;
+      S.lo[o0 + k * NN + j] = vl[k].x;
+      S.hi[o1 + k * NN + j] = vh[k].y;
+      S.lo[o1 + k * NN + j] = vl[k].y;
+      f0 = f0 && isfinite(vh[k].x);
+      f1 = f1 && isfinite(vh[k].y);
     }
-    if (active && !finite) atomicOr(status, SL_ST_NONFINITE);
+    const bool in0 = ex < P.kx && ey < P.ky, in1 = ex + 1 < P.kx && ey < P.ky;
+    if ((in0 && !f0) || (in1 && !f1)) atomicOr(status, SL_ST_NONFINITE);
   }
   __syncthreads();
 
@@ -397,9 +465,9 @@ __global__ void __launch_bounds__(Tile<NN, TX, TY>::NT)
     const int cnt = min(TX, P.kx - ex0);
     const int64_t g0 = ((int64_t)eyr * P.kx + ex0) * ND, g1 = g0 + (int64_t)cnt * ND;
     const int64_t A = floor4(g0 + 3), B = floor4(g1);
-    const int64_t a0 = s_a0[r];                   // global float G of this row is at r RS + (G - a0)
-    const float* rh = s_hi + r * RS;
-    const float* rl = s_lo + r * RS;
+    const int64_t a0 = S.a0[r];                   // global float G of this row is at r RS + (G - a0)
+    const float* rh = S.hi + r * RS;
+    const float* rl = S.lo + r * RS;
     if (A <= B) {
       const int nvec = (int)((B - A) >> 2);
       for (int v = tid; v < nvec; v += NT) {
@@ -428,10 +496,29 @@ __global__ void __launch_bounds__(Tile<NN, TX, TY>::NT)
 
 template <int NN, int TX, int TY>
 void launch(const Mixed2DConstParams& p, const float* tab, const float* in, float* out, unsigned* st, cudaStream_t s) {
+  Uni<NN> U;
+  auto two = [](float2* dst, const float* src, int n) {
+    for (int i = 0; i < n; ++i) dst[i] = make_float2(src[i], src[i]);
+  };
+  two(U.Rx, p.Rx, NN * NN);
+  two(U.Ry, p.Ry, NN * NN);
+  two(U.xix, p.xix, NN);
+  two(U.rox, p.rox, NN);
+  two(U.louty, p.louty, NN);
+  two(U.liny, p.liny, NN);
+  two(U.l0, p.l0, NN);
+  two(U.l1, p.l1, NN);
+  two(U.w, p.w, NN);
+  two(U.wh, p.wh, NN);
+  two(U.wl, p.wl, NN);
+  for (int i = 0; i < NN; ++i) U.nwh[i] = make_float2(-p.wh[i], -p.wh[i]);
+  const Head H{p.kx,  p.ky,  p.xw,   p.ys,   p.per_x, p.per_y, p.bnd, p.mass, p.mc,   p.refine, p.plane,
+               (float)p.ghost, (float)(p.ghost - (double)(float)p.ghost), p.sfx, p.sfy,
+               {p.al[0], p.al[1], p.al[2], p.al[3]}, p.o_kd, p.o_fx, p.o_fy, p.o_RyT, p.o_t, p.o_q, p.o_l0, p.o_l1, p.o_w, p.o_cm};
   dim3 grid((p.kx + TX - 1) / TX, (p.ky + TY - 1) / TY);
-  const size_t dyn = p.refine ? (size_t)Tile<NN, TX, TY>::NE * NN * 8 * sizeof(float) : 0;
-  if (dyn) allow_dynamic_smem((const void*)k_step2d_shared<NN, TX, TY>, dyn);
-  k_step2d_shared<NN, TX, TY><<<grid, Tile<NN, TX, TY>::NT, dyn, s>>>(p, tab, in, out, st);
+  constexpr size_t dyn = sizeof(Smem<NN, TX, TY>);
+  allow_dynamic_smem((const void*)k_step2d_shared<NN, TX, TY>, dyn);
+  k_step2d_shared<NN, TX, TY><<<grid, Tile<NN, TX, TY>::NT, dyn, s>>>(U, H, tab, in, out, st);
 }
 
 }  // namespace k2c

@@ -1,4 +1,4 @@
-// Host construction (long double) of the shared 2D step operator for a uniform mesh under a
+// Host construction (double; the tables are floats) of the shared 2D step operator for a uniform mesh under a
 // constant velocity (a, b): every element then sees the same advected geometry (Sec. 5.3), so the
 // remap (eq. 5.4, separable: A_y (x) A_x), the face traces (eq. 2dx/2dy_bnd_interpolate), the
 // upwind values (eq. 4.12a), the mass target (eq. remap_mass with the RK quadrature of the face
@@ -14,25 +14,23 @@
 // row is w (x) w, so the correction costs five products per node.
 #include <algorithm>
 #include <cmath>
-#include <map>
 
 #include "sl_internal.h"
 
 namespace sl {
 namespace {
-using ld = long double;
 
-std::vector<ld> basis_at(const std::vector<ld>& nodes, ld z) {
-  const int n = (int)nodes.size();
-  std::vector<ld> v(n, 1.0L);
-  for (int j = 0; j < n; ++j)
-    for (int m = 0; m < n; ++m)
-      if (m != j) v[j] *= (z - nodes[m]) / (nodes[j] - nodes[m]);
-  return v;
-}
+using vec = std::vector<double>;
+
+// distinct stage times of the RK orders 1-4 and their summed weights
+const int ds_n[5] = {0, 1, 2, 3, 3};
+const double ds_c[5][3] = {{}, {0.0}, {0.0, 1.0}, {0.0, 0.5, 1.0}, {0.0, 0.5, 1.0}};
+const double ds_b[5][3] = {{}, {1.0}, {0.5, 0.5}, {1.0 / 6, 2.0 / 3, 1.0 / 6}, {1.0 / 6, 2.0 / 3, 1.0 / 6}};
 
 }  // namespace
 
+// A first step pays for this construction, so it is O(n^3): the outflow-flux functionals are sums of a few
+// outer products, and (C C^T)^+ comes with the fit operators.
 bool build_mixed2d_const(const sl_ctx* c, double a, double b, double dt, unsigned cons, int rk,
                          std::vector<float>& buf, Mixed2DConstParams& P, std::string& err) {
   const int n = c->n, nd = n * n;
@@ -40,46 +38,47 @@ bool build_mixed2d_const(const sl_ctx* c, double a, double b, double dt, unsigne
   const double hx = (c->mesh.x1 - c->mesh.x0) / c->mesh.kx, hy = (c->mesh.y1 - c->mesh.y0) / c->mesh.ky;
   if (a == 0.0 || b == 0.0) { err = "the 2D shared-operator path needs both velocity components non-zero"; return false; }
   if (cons & SL_C_ENERGY) { err = "energy is applied by the general 2D mixed path"; return false; }
-  std::vector<ld> xi(B.xi.begin(), B.xi.end()), w(B.w.begin(), B.w.end());
-  const ld dx = (ld)a * dt / hx, dy = (ld)b * dt / hy;
+  const vec& w = B.w;
+  const double dx = a * dt / hx, dy = b * dt / hy;
   // remap matrices R[l][q] = l_q(xi_l - shift)
-  std::vector<ld> Rx(nd), Ry(nd);
+  vec Rx(nd), Ry(nd);
   for (int l = 0; l < n; ++l) {
-    std::vector<ld> vx = basis_at(xi, xi[l] - dx), vy = basis_at(xi, xi[l] - dy);
-    for (int q = 0; q < n; ++q) { Rx[l * n + q] = vx[q]; Ry[l * n + q] = vy[q]; }
+    basis_row(B, B.xi[l], -dx, Rx.data() + l * n);
+    basis_row(B, B.xi[l], -dy, Ry.data() + l * n);
   }
   const bool xw = a > 0.0, ys = b > 0.0;       // x-upwind neighbour is W (else E); y-upwind is S (else N)
-  std::vector<ld> l0 = basis_at(xi, 0.0L), l1 = basis_at(xi, 1.0L);
-  const std::vector<ld>& lin_x = xw ? l0 : l1;
-  const std::vector<ld>& lout_x = xw ? l1 : l0;
-  const std::vector<ld>& lin_y = ys ? l0 : l1;
-  const std::vector<ld>& lout_y = ys ? l1 : l0;
-  std::vector<ld> r_ox(n, 0.0L), r_oy(n, 0.0L);
+  const vec &l0 = B.l0, &l1 = B.l1;
+  const vec& lin_x = xw ? l0 : l1;
+  const vec& lout_x = xw ? l1 : l0;
+  const vec& lin_y = ys ? l0 : l1;
+  const vec& lout_y = ys ? l1 : l0;
+  vec r_ox(n, 0.0), r_oy(n, 0.0);
   for (int q = 0; q < n; ++q)
     for (int i = 0; i < n; ++i) {
       r_ox[q] += Rx[i * n + q] * lout_x[i];
       r_oy[q] += Ry[i * n + q] * lout_y[i];
     }
   // outflow-face flux functionals (mass): Kx[m][l] = |a| hy sum_s b_s sum_q w_q l_m(eta_q - c dy) l_l(xo - c dx)
-  static const double rkb[5][4] = {{}, {1.0}, {0.5, 0.5}, {1.0 / 6, 2.0 / 3, 1.0 / 6}, {1.0 / 6, 1.0 / 3, 1.0 / 3, 1.0 / 6}};
-  static const double rkc[5][4] = {{}, {0.0}, {0.0, 1.0}, {0.0, 0.5, 1.0}, {0.0, 0.5, 0.5, 1.0}};
-  std::map<double, ld> stages;
-  for (int s = 0; s < rk; ++s) stages[rkc[rk][s]] += (ld)rkb[rk][s];
-  std::vector<ld> Kx(nd, 0.0L), Ky(nd, 0.0L);
-  const ld xo = xw ? 1.0L : 0.0L, yo = ys ? 1.0L : 0.0L;
-  for (auto& kv : stages) {
-    const ld cs = kv.first, bs = kv.second;
-    std::vector<ld> ex = basis_at(xi, xo - cs * dx), ey = basis_at(xi, yo - cs * dy);
+  vec Kx(nd, 0.0), Ky(nd, 0.0);
+  const double xo = xw ? 1.0 : 0.0, yo = ys ? 1.0 : 0.0;
+  for (int s = 0; s < ds_n[rk]; ++s) {
+    const double cs = ds_c[rk][s], bs = ds_b[rk][s];
+    vec ex(n), ey(n), t(n), wx(n, 0.0), wy(n, 0.0);
+    basis_row(B, xo, -cs * dx, ex.data());
+    basis_row(B, yo, -cs * dy, ey.data());
     for (int q = 0; q < n; ++q) {
-      std::vector<ld> ty = basis_at(xi, xi[q] - cs * dy), tx = basis_at(xi, xi[q] - cs * dx);
-      for (int m = 0; m < n; ++m)
-        for (int l = 0; l < n; ++l) {
-          Kx[m * n + l] += std::fabs((ld)a) * hy * bs * w[q] * ty[m] * ex[l];
-          Ky[m * n + l] += std::fabs((ld)b) * hx * bs * w[q] * ey[m] * tx[l];
-        }
+      basis_row(B, B.xi[q], -cs * dy, t.data());
+      for (int m = 0; m < n; ++m) wy[m] += w[q] * t[m];
+      basis_row(B, B.xi[q], -cs * dx, t.data());
+      for (int m = 0; m < n; ++m) wx[m] += w[q] * t[m];
     }
+    for (int m = 0; m < n; ++m)
+      for (int l = 0; l < n; ++l) {
+        Kx[m * n + l] += std::fabs(a) * hy * bs * wy[m] * ex[l];
+        Ky[m * n + l] += std::fabs(b) * hx * bs * ey[m] * wx[l];
+      }
   }
-  const ld lam = (ld)dt / ((ld)hx * hy);
+  const double lam = dt / (hx * hy);
   // rows of the hard fit: W (n), E (n), S (n), N (n), mass (1) -- see make_fit_2d
   const FitOps& F = c->fit[cons & 3u][0];
   const int m = F.m;
@@ -92,14 +91,10 @@ bool build_mixed2d_const(const sl_ctx* c, double a, double b, double dt, unsigne
   }
   if (mass) cols.push_back(bnd ? 4 * n : 0);
   const int mc = (int)cols.size();
-  // (C C^T)^+ = (C+)^T C+, restricted to the kept columns: G[r][k]
-  std::vector<ld> G((size_t)m * mc, 0.0L);
+  // (C C^T)^+ restricted to the kept columns: G[r][k]
+  vec G((size_t)m * mc, 0.0);
   for (int r = 0; r < m; ++r)
-    for (int k = 0; k < mc; ++k) {
-      ld acc = 0.0L;
-      for (int q = 0; q < nd; ++q) acc += (ld)F.Cpinv[q * m + r] * (ld)F.Cpinv[q * m + cols[k]];
-      G[(size_t)r * mc + k] = acc;
-    }
+    for (int k = 0; k < mc; ++k) G[(size_t)r * mc + k] = F.Gp[(size_t)r * m + cols[k]];
   P = Mixed2DConstParams{};
   P.n = n;
   P.kx = c->mesh.kx;
@@ -122,9 +117,9 @@ bool build_mixed2d_const(const sl_ctx* c, double a, double b, double dt, unsigne
       P.Rxp[q][i] = make_float2(P.Rx[2 * q * n + i], P.Rx[(2 * q + 1) * n + i]);
       P.Ryp[q][i] = make_float2(P.Ry[2 * q * n + i], P.Ry[(2 * q + 1) * n + i]);
     }
-  std::vector<ld> wxr(n, 0.0L), wyr(n, 0.0L);   // R_x^T w, R_y^T w: mass of psihat is wyr^T psi wxr
+  vec wxr(n, 0.0), wyr(n, 0.0);   // R_x^T w, R_y^T w: mass of psihat is wyr^T psi wxr
   for (int p = 0; p < n; ++p) {
-    ld xi_in = 0.0L;
+    double xi_in = 0.0;
     for (int l = 0; l < n; ++l) {
       xi_in += Rx[l * n + p] * lin_x[l];
       wxr[p] += Rx[l * n + p] * w[l];
@@ -143,41 +138,91 @@ bool build_mixed2d_const(const sl_ctx* c, double a, double b, double dt, unsigne
     for (int k = 0; k < mc; ++k) P.gm[k] = (float)G[(size_t)rm * mc + k];
   }
   buf.clear();
-  auto put = [&](const std::vector<ld>& v) {
+  auto put = [&](const vec& v) {
     size_t off = buf.size();
-    for (ld x : v) buf.push_back((float)x);
+    for (double x : v) buf.push_back((float)x);
     return (int)off;
   };
   // tables a thread reads by its own row j are stored [other index][j], so that the n threads of
   // an element read n consecutive floats
-  auto transpose = [n](const std::vector<ld>& M) {
-    std::vector<ld> T(M.size());
+  auto transpose = [n](const vec& M) {
+    vec T(M.size());
     for (int r = 0; r < n; ++r)
       for (int q = 0; q < n; ++q) T[q * n + r] = M[r * n + q];
     return T;
   };
   // mass residual functionals (reference measure): own psi, x-neighbour psi_X (row j of each) and
   // y-neighbour psi_Y (column j); the mass of psihat is folded into the own functional
-  std::vector<ld> Ks(nd), Kxl(nd), Kyl(nd);
+  vec Ks(nd), Kxl(nd), Kyl(nd), Kd(nd);
   for (int j = 0; j < n; ++j)
     for (int i = 0; i < n; ++i) {
       const int k = j * n + i;
       Ks[k] = w[j] * w[i] - lam * (Kx[k] + Ky[k]) - wyr[j] * wxr[i];
+      Kd[k] = w[j] * w[i] - wyr[j] * wxr[i];
       Kxl[k] = lam * Kx[k];
       Kyl[k] = lam * Ky[k];
     }
   P.o_ks = put(transpose(Ks));
   P.o_kx = put(transpose(Kxl));
   P.o_ky = put(Kyl);                             // column j of psi_Y: entry [m][j]
+  P.o_kd = put(transpose(Kd));
   P.o_RxT = put(transpose(Rx));
   P.o_RyT = put(transpose(Ry));
   // face rows of G as Gt[(f * mc + k) * n + j] = G[f n + j][k], f = W, E, S, N
   if (bnd) {
-    std::vector<ld> Gt((size_t)4 * mc * n);
+    vec Gt((size_t)4 * mc * n);
     for (int f = 0; f < 4; ++f)
       for (int k = 0; k < mc; ++k)
         for (int j = 0; j < n; ++j) Gt[((size_t)f * mc + k) * n + j] = G[(size_t)(f * n + j) * mc + k];
     P.o_g = put(Gt);
+  }
+  {
+    // orthonormal basis Q of span{l0, l1, w} (twice orthogonalised; a dependent vector leaves a zero column)
+    vec Q(3 * n, 0.0), T((size_t)13 * (2 * n + 1), 0.0);
+    const vec* span[3] = {&l0, &l1, &w};
+    for (int c = 0; c < 3; ++c) {
+      vec v = *span[c];
+      double v0 = 0.0, v1 = 0.0;
+      for (double x : v) v0 += x * x;
+      for (int pass = 0; pass < 2; ++pass)
+        for (int e = 0; e < c; ++e) {
+          double d = 0.0;
+          for (int i = 0; i < n; ++i) d += Q[e * n + i] * v[i];
+          for (int i = 0; i < n; ++i) v[i] -= d * Q[e * n + i];
+        }
+      for (double x : v) v1 += x * x;
+      if (v1 > 1e-20 * v0)
+        for (int i = 0; i < n; ++i) Q[c * n + i] = v[i] / std::sqrt(v1);
+    }
+    // on the complement of the span opposite faces couple by [a b; b a]
+    double a2 = 0.0, b2 = 0.0;
+    for (int i = 0; i < n; ++i) {
+      a2 += l0[i] * l0[i];
+      b2 += l0[i] * l1[i];
+    }
+    const int fx = xw ? 0 : 1, fy = ys ? 2 : 3, W2 = 2 * n + 1;
+    for (int f = 0; f < 4; ++f) {
+      const bool in = f == fx || f == fy;
+      const double al = bnd ? (in ? a2 : -b2) / (a2 * a2 - b2 * b2) : 0.0;
+      P.al[f] = (float)al;
+      for (int c = 0; c < 3 && bnd; ++c)
+        for (int k = 0; k < mc; ++k) {
+          double t = 0.0;
+          for (int j = 0; j < n; ++j)
+            t += Q[c * n + j] * (G[(size_t)(f * n + j) * mc + k] - (k == (f < 2 ? j : n + j) ? al : 0.0));
+          T[(size_t)(3 * f + c) * W2 + k] = t;
+        }
+    }
+    if (mass && bnd)
+      for (int k = 0; k < mc; ++k) T[(size_t)12 * W2 + k] = G[(size_t)4 * n * mc + k];
+    if (mass && !bnd) T[12] = G[0];
+    P.o_t = put(T);
+    P.o_q = put(Q);
+    for (int i = 0; i < n; ++i) {
+      P.louty[i] = (float)lout_y[i];
+      P.wh[i] = (float)w[i];
+      P.wl[i] = (float)(w[i] - (double)P.wh[i]);
+    }
   }
   P.o_l0 = put(l0);
   P.o_l1 = put(l1);
@@ -186,24 +231,14 @@ bool build_mixed2d_const(const sl_ctx* c, double a, double b, double dt, unsigne
   // float functional of its own values (lam Kx, lam Ky), evaluated alike by the element and by its
   // downstream neighbour; w (x) w in float-float; the mass column of C+
   // the refinement moves mass along C+ e_m, which keeps the face rows only when C C+ e_m = e_m
-  bool indep = false;
-  if (mass) {
-    const int rm = bnd ? 4 * n : 0;
-    ld dev = 0.0L;
-    for (int k = 0; k < m; ++k) {
-      ld acc = 0.0L;
-      for (int q = 0; q < nd; ++q) acc += (ld)F.C[(size_t)k * nd + q] * (ld)F.Cpinv[(size_t)q * m + rm];
-      dev = std::max(dev, std::fabs(acc - (k == rm ? 1.0L : 0.0L)));
-    }
-    indep = dev < 1e-9L;
-  }
+  const bool indep = mass && F.last_free;
   P.refine = indep ? 1 : 0;
-  if (indep) {
-    std::vector<ld> fx(nd), fy(nd), wh(nd), wl(nd), cm(nd);
+  if (mass) {
+    vec fx(nd), fy(nd);
     float sfx = 0.0f, sfy = 0.0f;
     for (int k = 0; k < nd; ++k) {
-      fx[k] = (ld)(float)(lam * Kx[k]);
-      fy[k] = (ld)(float)(lam * Ky[k]);
+      fx[k] = (double)(float)(lam * Kx[k]);
+      fy[k] = (double)(float)(lam * Ky[k]);
     }
     // the sums in the order the kernel forms a row's partial sums and then adds the rows
     for (int j = 0; j < n; ++j) {
@@ -217,16 +252,19 @@ bool build_mixed2d_const(const sl_ctx* c, double a, double b, double dt, unsigne
     }
     P.sfx = sfx;
     P.sfy = sfy;
+    P.o_fx = put(transpose(fx));
+    P.o_fy = put(transpose(fy));
+  }
+  if (indep) {
+    vec wh(nd), wl(nd), cm(nd);
     const int rmass = bnd ? 4 * n : 0;
     for (int j = 0; j < n; ++j)
       for (int i = 0; i < n; ++i) {
         const double v = B.w[i] * B.w[j];
-        wh[j * n + i] = (ld)(float)v;
-        wl[j * n + i] = (ld)(float)(v - (double)(float)v);
-        cm[j * n + i] = (ld)F.Cpinv[(size_t)(j * n + i) * m + rmass];
+        wh[j * n + i] = (double)(float)v;
+        wl[j * n + i] = (double)(float)(v - (double)(float)v);
+        cm[j * n + i] = (double)F.Cpinv[(size_t)(j * n + i) * m + rmass];
       }
-    P.o_fx = put(transpose(fx));
-    P.o_fy = put(transpose(fy));
     P.o_wh = put(transpose(wh));
     P.o_wl = put(transpose(wl));
     P.o_cm = put(cm);                          // [k][j]: node (j, k) of column j at k n + j

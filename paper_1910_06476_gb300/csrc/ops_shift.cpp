@@ -11,15 +11,6 @@ namespace sl {
 
 namespace {
 
-void basis_row(const Basis1D& B, double z0, double dz, double* out) {
-  for (int l = 0; l < B.n; ++l) {
-    double p = B.lam[l];
-    for (int k = 0; k < B.n; ++k)
-      if (k != l) p *= (z0 - B.xi[k]) + dz;
-    out[l] = p;
-  }
-}
-
 // distinct stage times of the RK orders 1-4 and their summed weights (RK4's two c = 1/2 stages coincide)
 const int ds_n[5] = {0, 1, 2, 3, 3};
 const double ds_c[5][3] = {{}, {0.0}, {0.0, 1.0}, {0.0, 0.5, 1.0}, {0.0, 0.5, 1.0}};

@@ -38,6 +38,9 @@ struct Basis1D {
 
 Basis1D make_basis(int n, int basis);
 
+// Lagrange basis values at z0 + dz, out[l], differences formed as (z0 - xi_k) + dz
+void basis_row(const Basis1D& B, double z0, double dz, double* out);
+
 // Dense row-major operators of the constrained fit for one constraint set.
 //   hard: phi_L = phihat + Cpinv (d - C phihat);  q = a - Cpinv (C a)
 //   soft: phi_L = S phihat + SCt d;                q = S a
@@ -47,6 +50,8 @@ struct FitOps {
   std::vector<double> Cpinv;             // nd x m (hard)
   std::vector<double> S;                 // nd x nd (soft)
   std::vector<double> SCt;               // nd x m (soft)
+  std::vector<double> Gp;                // m x m (hard): (C C^T)^+
+  bool last_free = false;                // (hard) the last row is independent of the others: C C^+ e_m = e_m
 };
 
 // 1D constraint rows for a mask (left face, right face, mass in the reference measure).
@@ -223,6 +228,14 @@ struct Mixed2DConstParams {
   int refine;
   float sfx, sfy;
   int o_fx, o_fy, o_wh, o_wl, o_cm;
+  int o_kd;                                 // w (x) w - (R^T w) (x) (R^T w): own mass less the mass of psihat
+  // (C C^T)^+ by structure: s_F = al_F r + Q c_F; o_q: Q ([3][n], orthonormal basis of span{l0, l1, w}, zero
+  // columns where the span is smaller), o_t: the 13 coefficients' rows ([13][2 n + 1] over x residuals, y
+  // residuals, mass residual; three per face W, E, S, N, then the mass row of (C C^T)^+)
+  float al[4];
+  int o_q, o_t;
+  float louty[NMAX];                        // basis on the y-outflow face
+  float wh[NMAX], wl[NMAX];                 // quadrature weights as float-float
 };
 bool build_mixed2d_const(const sl_ctx* c, double a, double b, double dt, unsigned cons, int rk,
                          std::vector<float>& buf, Mixed2DConstParams& P, std::string& err);

@@ -160,6 +160,15 @@ Basis1D make_basis(int n, int basis) {
   return b;
 }
 
+void basis_row(const Basis1D& B, double z0, double dz, double* out) {
+  for (int l = 0; l < B.n; ++l) {
+    double p = B.lam[l];
+    for (int k = 0; k < B.n; ++k)
+      if (k != l) p *= (z0 - B.xi[k]) + dz;
+    out[l] = p;
+  }
+}
+
 void finish_fit(FitOps& f, bool soft) {
   const int m = f.m, nd = f.nd;
   if (m == 0) {                    // no linear rows: phi_L = phihat, q = a
@@ -195,6 +204,14 @@ void finish_fit(FitOps& f, bool soft) {
         for (int i = 0; i < m; ++i) s += C[i * nd + r] * Gp[i * m + j];
         f.Cpinv[r * m + j] = (double)s;
       }
+    f.Gp.assign(Gp.begin(), Gp.end());
+    ld dev = 0.0L;                               // C C^+ e_m against e_m
+    for (int k = 0; k < m; ++k) {
+      ld s = 0.0L;
+      for (int i = 0; i < m; ++i) s += G[k * m + i] * Gp[i * m + m - 1];
+      dev = std::max(dev, std::fabs(s - (k == m - 1 ? 1.0L : 0.0L)));
+    }
+    f.last_free = dev < 1e-9L;
   } else {
     std::vector<ld> A(nd * nd, 0.0L);
     for (int r = 0; r < nd; ++r) A[r * nd + r] = 1.0L;
