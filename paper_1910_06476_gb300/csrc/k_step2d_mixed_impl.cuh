@@ -38,6 +38,14 @@
 // while h <= 1/4, so that |pi h d| <= pi / 4 where ten terms are exact to 1e-9; coarser meshes evaluate
 // sinpi and cospi directly).  cos(pi t / T) is taken once per element at the stage-time fractions 0,
 // 1/4, 1/2, 3/4, 1 of the step, which cover the RK schemes and their backward feet.
+// Bound by instruction issue (63 % / 70 % of the issue slots in the two phases; FMA pipe 40 % / 30 %, HBM 4 %).
+// Measured (one GB300), 512 x 512 elements of n = 8, swirl, every constraint: phase 1 757 -> 699 us (607 -> 544 M
+// warp instructions), phase 2 597 -> 365 us (353 -> 236 M).  What that took: no FP64 instruction (element corners
+// in float-float, per-problem parameters from the host), the upwind side of each face point formed once in
+// phase 1 from the tabulated sines, the pseudo-inverse read as pairs with a thread's two nodes side by side and
+// skipped for faces whose residual vanishes, one evaluation for all tabulated sines, maxima by one integer
+// reduction, reductions that share a barrier merged, the preconditioner's passes as dot products of rows in
+// 16-byte vectors at a conflict-free stride, the traces and the face fluxes in one pass over the face points.
 #include <type_traits>
 
 #include "k_map2d.cuh"
@@ -74,6 +82,10 @@ __device__ __forceinline__ ff lref(float r0, float gx, float gy, float a, float 
   const float t = fmaf(gx, a, __fmul_rn(gy, b));
   return two_sum(r0, t);
 }
+// the same at two points at once
+__device__ __forceinline__ ff2 lref2(float r0, float gx, float gy, float2 a, float2 b) {
+  return two_sum2(dup(r0), __ffma2_rn(dup(gx), a, __fmul2_rn(dup(gy), b)));
+}
 
 // ------------------------------------------------------------------ groups of warps
 template <int NN>
@@ -84,15 +96,20 @@ struct Shape {
   static constexpr int EPC = G == 1 ? 8 : G == 2 ? 4 : G <= 4 ? 2 : 1;   // element groups per CTA
   static constexpr int NT = GT * EPC;
   static constexpr int NP = (NN + 3) & ~3;                 // row stride of psihat and psi^n (16 bytes)
-  static constexpr int RS = NN | 1;                        // odd row stride of the preconditioner rows
-  static constexpr int MINB = NN <= 12 ? 2 : 1;            // resident CTAs asked of the compiler: phase 1
-  static constexpr int MINB2 = NN <= 8 ? 3 : NN <= 12 ? 2 : 1;   // phase 2 (measured: 3 beats 2 at n = 8)
+  // row stride of the preconditioner tables: the rows that lanes read side by side, as 16-byte vectors, start
+  // in different banks
+  static constexpr int RP = NP + (NP % 8 == 0 ? 4 : 0);
+  // resident CTAs asked of the compiler.  Phase 1 at three (80 registers) spills: the large swirl took 17.0 ms
+  // instead of 15.4; below two, n >= 13 ran 6-8 warps per SM.  Phase 2 fits four since the far-neighbour
+  // interpolation is out of line
+  static constexpr int MINB = 2;
+  static constexpr int MINB2 = NN <= 16 ? 4 : 3;
 };
 
 template <int G>
 struct Grp {
   int t, lane, w, slot;
-  float* red;                                              // 4 G floats: two buffers of a pair per warp
+  float* red;                                              // 8 G floats: two buffers of four values per warp
   int rb;
   __device__ __forceinline__ void sync() const {
     if (G == 1) __syncwarp();
@@ -104,7 +121,7 @@ struct Grp {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     if (G == 1) return v;
-    float* r = red + rb * 2 * G;
+    float* r = red + rb * 4 * G;
     rb ^= 1;
     if (lane == 0) r[w] = v;
     sync();
@@ -116,11 +133,13 @@ struct Grp {
   __device__ __forceinline__ float2 sum2(float a, float b) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-      a += __shfl_xor_sync(0xffffffffu, a, o);
-      b += __shfl_xor_sync(0xffffffffu, b, o);
+      const float2 v = __fadd2_rn(make_float2(a, b), make_float2(__shfl_xor_sync(0xffffffffu, a, o),
+                                                                 __shfl_xor_sync(0xffffffffu, b, o)));
+      a = v.x;
+      b = v.y;
     }
     if (G == 1) return make_float2(a, b);
-    float* r = red + rb * 2 * G;
+    float* r = red + rb * 4 * G;
     rb ^= 1;
     if (lane == 0) { r[w] = a; r[G + w] = b; }
     sync();
@@ -129,32 +148,93 @@ struct Grp {
     for (int k = 0; k < G; ++k) { sa += r[k]; sb += r[G + k]; }
     return make_float2(sa, sb);
   }
+  // maximum of non-negative values: their bits order like the values (one warp instruction); NaN, whose bits
+  // are above infinity's, wins
   __device__ __forceinline__ float max(float v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+    v = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(v)));
     if (G == 1) return v;
-    float* r = red + rb * 2 * G;
+    float* r = red + rb * 4 * G;
     rb ^= 1;
     if (lane == 0) r[w] = v;
     sync();
-    float s = 0.0f;
+    unsigned s = 0u;
 #pragma unroll
-    for (int k = 0; k < G; ++k) s = fmaxf(s, r[k]);
-    return s;
+    for (int k = 0; k < G; ++k) s = ::max(s, __float_as_uint(r[k]));
+    return __uint_as_float(s);
   }
+  // two or three sums and a maximum of non-negative values in one pass (one barrier between the warps)
+  __device__ __forceinline__ void sum3max(float& a, float& b, float& c, float& m, bool three) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const float2 v = __fadd2_rn(make_float2(a, b), make_float2(__shfl_xor_sync(0xffffffffu, a, o),
+                                                                 __shfl_xor_sync(0xffffffffu, b, o)));
+      a = v.x;
+      b = v.y;
+      if (three) c += __shfl_xor_sync(0xffffffffu, c, o);
+    }
+    m = __uint_as_float(__reduce_max_sync(0xffffffffu, __float_as_uint(m)));
+    if (G == 1) return;
+    float* r = red + rb * 4 * G;
+    rb ^= 1;
+    if (lane == 0) { r[w] = a; r[G + w] = b; r[2 * G + w] = c; r[3 * G + w] = m; }
+    sync();
+    a = b = c = 0.0f;
+    unsigned mx = 0u;
+#pragma unroll
+    for (int k = 0; k < G; ++k) {
+      a += r[k];
+      b += r[G + k];
+      if (three) c += r[2 * G + k];
+      mx = ::max(mx, __float_as_uint(r[3 * G + k]));
+    }
+    m = __uint_as_float(mx);
+  }
+  // float-float sum: the high parts by two-sums, their errors and the low parts in one float (symmetric at
+  // every level, so every lane gets the same bits), renormalised once
   __device__ __forceinline__ ff ffsum(ff v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-      ff u;
-      u.hi = __shfl_xor_sync(0xffffffffu, v.hi, o);
-      u.lo = __shfl_xor_sync(0xffffffffu, v.lo, o);
-      v = ff_add(v, u);
+      const float uh = __shfl_xor_sync(0xffffffffu, v.hi, o), ul = __shfl_xor_sync(0xffffffffu, v.lo, o);
+      const ff s = two_sum(v.hi, uh);
+      v.hi = s.hi;
+      v.lo = __fadd_rn(__fadd_rn(v.lo, ul), s.lo);
     }
+    v = fast_two_sum(v.hi, v.lo);
     if (G == 1) return v;
-    float* r = red + rb * 2 * G;
+    float* r = red + rb * 4 * G;
     rb ^= 1;
     if (lane == 0) { r[w] = v.hi; r[G + w] = v.lo; }
     sync();
+    return ffjoin(r);
+  }
+  // the same, with two plain sums in the same pass
+  __device__ __forceinline__ ff ffsum_sum2(ff v, float& a, float& b) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      const float uh = __shfl_xor_sync(0xffffffffu, v.hi, o), ul = __shfl_xor_sync(0xffffffffu, v.lo, o);
+      const ff s = two_sum(v.hi, uh);
+      v.hi = s.hi;
+      v.lo = __fadd_rn(__fadd_rn(v.lo, ul), s.lo);
+      const float2 u = __fadd2_rn(make_float2(a, b), make_float2(__shfl_xor_sync(0xffffffffu, a, o),
+                                                                 __shfl_xor_sync(0xffffffffu, b, o)));
+      a = u.x;
+      b = u.y;
+    }
+    v = fast_two_sum(v.hi, v.lo);
+    if (G == 1) return v;
+    float* r = red + rb * 4 * G;
+    rb ^= 1;
+    if (lane == 0) { r[w] = v.hi; r[G + w] = v.lo; r[2 * G + w] = a; r[3 * G + w] = b; }
+    sync();
+    a = b = 0.0f;
+#pragma unroll
+    for (int k = 0; k < G; ++k) {
+      a += r[2 * G + k];
+      b += r[3 * G + k];
+    }
+    return ffjoin(r);
+  }
+  __device__ __forceinline__ ff ffjoin(const float* r) const {
     ff s = {r[0], r[G]};
 #pragma unroll
     for (int k = 1; k < G; ++k) s = ff_add(s, ff{r[k], r[G + k]});
@@ -292,10 +372,12 @@ __device__ __forceinline__ void vel_swirl_tab(const VelElem& V, float Sx, float 
   const float sx = fmaf(Sx, ctt, Cx * st), cx = fmaf(Cx, ctt, -Sx * st);
   small_sincos(V.pihy * dy, V.shortser, st, ctt);
   const float sy = fmaf(Sy, ctt, Cy * st), cy = fmaf(Cy, ctt, -Sy * st);
-  u = sx * sx * (2.0f * sy * cy) * ct * V.ihx;
-  v = -sy * sy * (2.0f * sx * cx) * ct * V.ihy;
+  const float p = sx * sy;
+  u = (p * (sx * cy)) * (2.0f * ct * V.ihx);
+  v = (p * (sy * cx)) * (-2.0f * ct * V.ihy);
 }
 
+// The displacement starts at zero, so the first stage is the base point itself.
 // TAB: the velocity is the swirl from the tabulated sines (chosen once per element)
 template <int RK, bool TAB>
 __device__ __forceinline__ void rk_disp_t(const VelElem& V, float bx, float by, float Sx, float Cx, float Sy, float Cy,
@@ -304,7 +386,7 @@ __device__ __forceinline__ void rk_disp_t(const VelElem& V, float bx, float by, 
   float kx[T::S], ky[T::S];
 #pragma unroll
   for (int s = 0; s < T::S; ++s) {
-    float xs = dx, ys = dy;
+    float xs = 0.0f, ys = 0.0f;
 #pragma unroll
     for (int j = 0; j < s; ++j)
       if (T::a(s, j) != 0.0f) {
@@ -312,7 +394,11 @@ __device__ __forceinline__ void rk_disp_t(const VelElem& V, float bx, float by, 
         ys = fmaf(h * T::a(s, j), ky[j], ys);
       }
     const int ci = __float2int_rn(4.0f * fmaf(T::c(s), fstep, f0));
-    if (TAB) vel_swirl_tab(V, Sx, Cx, Sy, Cy, xs, ys, ctab[ci], kx[s], ky[s]);
+    if (TAB && s == 0) {
+      const float p = Sx * Sy;
+      kx[0] = (p * (Sx * Cy)) * (2.0f * ctab[ci] * V.ihx);
+      ky[0] = (p * (Sy * Cx)) * (-2.0f * ctab[ci] * V.ihy);
+    } else if (TAB) vel_swirl_tab(V, Sx, Cx, Sy, Cy, xs, ys, ctab[ci], kx[s], ky[s]);
     else vel_at(V, bx, by, Sx, Cx, Sy, Cy, xs, ys, ctab[ci], kx[s], ky[s]);
   }
   float sx = 0.0f, sy = 0.0f;
@@ -321,8 +407,8 @@ __device__ __forceinline__ void rk_disp_t(const VelElem& V, float bx, float by, 
     sx = fmaf(T::b(s), kx[s], sx);
     sy = fmaf(T::b(s), ky[s], sy);
   }
-  dx = fmaf(h, sx, dx);
-  dy = fmaf(h, sy, dy);
+  dx = h * sx;
+  dy = h * sy;
 }
 
 __device__ __forceinline__ void rk_disp(const VelElem& V, int rk, float bx, float by, float Sx, float Cx, float Sy,
@@ -384,7 +470,7 @@ __device__ __forceinline__ void rk_disp2_t(const VelElem& V, float2 bx, float2 b
   float2 kx[T::S], ky[T::S];
 #pragma unroll
   for (int s = 0; s < T::S; ++s) {
-    float2 xs = dx, ys = dy;
+    float2 xs = bc2(0.0f), ys = bc2(0.0f);
 #pragma unroll
     for (int j = 0; j < s; ++j)
       if (T::a(s, j) != 0.0f) {
@@ -393,14 +479,19 @@ __device__ __forceinline__ void rk_disp2_t(const VelElem& V, float2 bx, float2 b
         ys = fma2(hj, ky[j], ys);
       }
     const float ct = ctab[__float2int_rn(4.0f * T::c(s))];
-    if (TAB) {
+    if (TAB && s == 0) {
+      const float2 p = mul2(Sx, Sy);
+      kx[0] = mul2(mul2(p, bc2(2.0f * ct * V.ihx)), mul2(Sx, Cy));
+      ky[0] = mul2(mul2(p, bc2(-2.0f * ct * V.ihy)), mul2(Sy, Cx));
+    } else if (TAB) {
       float2 st, ctt;
       small_sincos2(mul2(bc2(V.pihx), xs), V.shortser, st, ctt);
       const float2 sx = fma2(Sx, ctt, mul2(Cx, st)), cx = fma2(Cx, ctt, mul2(neg2(Sx), st));
       small_sincos2(mul2(bc2(V.pihy), ys), V.shortser, st, ctt);
       const float2 sy = fma2(Sy, ctt, mul2(Cy, st)), cy = fma2(Cy, ctt, mul2(neg2(Sy), st));
-      kx[s] = mul2(mul2(sx, sx), mul2(mul2(sy, cy), bc2(2.0f * ct * V.ihx)));
-      ky[s] = mul2(mul2(sy, sy), mul2(mul2(sx, cx), bc2(-2.0f * ct * V.ihy)));
+      const float2 p = mul2(sx, sy);
+      kx[s] = mul2(mul2(p, bc2(2.0f * ct * V.ihx)), mul2(sx, cy));
+      ky[s] = mul2(mul2(p, bc2(-2.0f * ct * V.ihy)), mul2(sy, cx));
     } else {
       vel_at2(V, bx, by, Sx, Cx, Sy, Cy, xs, ys, ct, kx[s], ky[s]);
     }
@@ -411,8 +502,8 @@ __device__ __forceinline__ void rk_disp2_t(const VelElem& V, float2 bx, float2 b
     sx = fma2(bc2(T::b(s)), kx[s], sx);
     sy = fma2(bc2(T::b(s)), ky[s], sy);
   }
-  dx = fma2(bc2(h), sx, dx);
-  dy = fma2(bc2(h), sy, dy);
+  dx = mul2(bc2(h), sx);
+  dy = mul2(bc2(h), sy);
 }
 
 // forward step over the whole step h = dt from t^n
@@ -516,24 +607,6 @@ __device__ __forceinline__ float row_dot(const float* row, const float (&b)[NN])
   return r;
 }
 
-// per-problem float parameters of a batch element (the FP64 geometry is already in P)
-__device__ __forceinline__ void batch_extra(const StepParams& P, const Map2D& M, Mixed2DExtra& X) {
-  if (!M.geo) return;
-  X.hx = (float)P.hx;
-  X.hy = (float)P.hy;
-  X.ihx = (float)(1.0 / P.hx);
-  X.ihy = (float)(1.0 / P.hy);
-  X.dt = (float)P.dt;
-  const double lam = P.dt / (P.hx * P.hy);
-  X.dt_area = (float)lam;
-  X.lam_hi = (float)lam;
-  X.lam_lo = (float)(lam - (double)X.lam_hi);
-  if (X.Tper != 0.0) {
-    X.tT = (float)(P.t / X.Tper);
-    X.dtT = (float)(P.dt / X.Tper);
-  }
-}
-
 __device__ __forceinline__ int nb_index(const StepParams& P, int ex, int ey, int face) {
   int jx = ex + (face == 0 ? -1 : face == 1 ? 1 : 0);
   int jy = ey + (face == 2 ? -1 : face == 3 ? 1 : 0);
@@ -546,31 +619,65 @@ __device__ __forceinline__ int nb_index(const StepParams& P, int ex, int ey, int
   return jy * P.kx + jx;
 }
 
-// the element of launch-list index k; copies its problem's geometry and step into P (batches)
+// sum_q a[q] b[q] of two shared rows (16-byte aligned, padded to 4): even and odd terms in the lanes of paired FMAs
 template <int NN>
-__device__ __forceinline__ Elem elem_at(StepParams& P, const Map2D& M, int64_t k) {
+__device__ __forceinline__ float dot_rows(const float* a, const float* b) {
+  const float4* ap = reinterpret_cast<const float4*>(a);
+  const float4* bp = reinterpret_cast<const float4*>(b);
+  float2 r2 = make_float2(0.0f, 0.0f);
+#pragma unroll
+  for (int q = 0; q < NN / 4; ++q) {
+    const float4 u = ap[q], v = bp[q];
+    r2 = __ffma2_rn(make_float2(u.x, u.y), make_float2(v.x, v.y), r2);
+    r2 = __ffma2_rn(make_float2(u.z, u.w), make_float2(v.z, v.w), r2);
+  }
+  float r = r2.x + r2.y;
+  if (NN % 4 != 0) {
+    const float4 u = ap[NN / 4], v = bp[NN / 4];
+    r = fmaf(u.x, v.x, r);
+    if (NN % 4 > 1) r = fmaf(u.y, v.y, r);
+    if (NN % 4 > 2) r = fmaf(u.z, v.z, r);
+  }
+  return r;
+}
+
+// the element of launch-list index k, and its problem's record (batches, else null)
+template <int NN>
+__device__ __forceinline__ Elem elem_at(const StepParams& P, const Map2D& M, int64_t k, const ProbGeom*& geo) {
   Elem E;
   E.g = M.list ? (int64_t)M.list[k] : k;
   E.gb = 0;
+  geo = nullptr;
+  int kx = P.kx;
   if (M.geo) {
-    const ProbGeom& G = M.geo[M.prob[E.g]];
-    P.kx = G.kx;
-    P.ky = G.ky;
-    for (int f = 0; f < 4; ++f) P.bc[f] = G.bc[f];
-    P.x0 = G.x0;
-    P.hx = G.hx;
-    P.y0 = G.y0;
-    P.hy = G.hy;
-    P.ghost = G.ghost;
-    P.t = G.t;
-    P.dt = G.dt;
-    E.gb = G.gbase;
+    geo = M.geo + M.prob[E.g];
+    kx = geo->kx;
+    E.gb = geo->gbase;
   }
   E.e = (int)(E.g - E.gb);
-  E.ex = E.e % P.kx;
-  E.ey = E.e / P.kx;
+  E.ey = E.e / kx;
+  E.ex = E.e - E.ey * kx;
   E.base = M.off ? M.off[E.g] : E.g * (NN * NN);
   return E;
+}
+
+// a problem's mesh and float parameters into P and X (batches)
+__device__ __forceinline__ void use_problem(const ProbGeom* G, StepParams& P, Mixed2DExtra& X) {
+  if (!G) return;
+  P.kx = G->kx;
+  P.ky = G->ky;
+  for (int f = 0; f < 4; ++f) P.bc[f] = G->bc[f];
+  P.ghost = G->ghost;
+  X.f = G->f;
+}
+
+// corner of element e along one direction, x0 + e h rounded to float, in float-float arithmetic (FP64
+// instructions would stall the element on the FP64 pipe); e < 2^24 or rounded once
+__device__ __forceinline__ float corner_of(float x0, float x0l, float h, float hl, int e) {
+  const float ef = (float)e, el = (float)(e - (int)ef);
+  const ff p = two_prod(ef, h);
+  const ff s = two_sum(x0, p.hi);
+  return __fadd_rn(s.hi, __fadd_rn(s.lo, __fadd_rn(fmaf(ef, hl, fmaf(el, h, p.lo)), x0l)));
 }
 
 __device__ __forceinline__ VelElem make_vel(const StepParams& P, const Mixed2DExtra& X, float x0, float y0) {
@@ -578,13 +685,13 @@ __device__ __forceinline__ VelElem make_vel(const StepParams& P, const Mixed2DEx
   V.kind = P.vel_kind;
   V.x0 = x0;
   V.y0 = y0;
-  V.hx = X.hx;
-  V.hy = X.hy;
-  V.ihx = X.ihx;
-  V.ihy = X.ihy;
-  V.pihx = 3.14159265358979f * X.hx;
-  V.pihy = 3.14159265358979f * X.hy;
-  V.direct = !(X.hx <= 0.25f && X.hy <= 0.25f);
+  V.hx = X.f.hx;
+  V.hy = X.f.hy;
+  V.ihx = X.f.ihx;
+  V.ihy = X.f.ihy;
+  V.pihx = 3.14159265358979f * X.f.hx;
+  V.pihy = 3.14159265358979f * X.f.hy;
+  V.direct = !(X.f.hx <= 0.25f && X.f.hy <= 0.25f);
   V.shortser = V.pihx <= 0.02f && V.pihy <= 0.02f;
   V.a = X.a;
   V.b = X.b;
@@ -607,46 +714,57 @@ struct Trig {
 template <int NN, int G>
 __device__ __forceinline__ void trig_setup(const Grp<G>& g, const VelElem& V, const Mixed2DExtra& X, const float* xi,
                                            Trig<NN>& T) {
-  const int t = g.t;
+  // every lane evaluates one coordinate (a branch per kind of coordinate would run the evaluation four times)
   if (V.kind == SL_VEL_SWIRL) {
-    if (t < NN) sincospif(fmaf(V.hx, xi[t], V.x0), &T.n[0][t], &T.n[1][t]);
-    else if (t < 2 * NN) sincospif(fmaf(V.hy, xi[t - NN], V.y0), &T.n[2][t - NN], &T.n[3][t - NN]);
-    else if (t < 2 * NN + 4) {
-      const int k = t - 2 * NN;
-      const float z = k < 2 ? V.x0 + (k == 1 ? V.hx : 0.0f) : V.y0 + (k == 3 ? V.hy : 0.0f);
-      sincospif(z, &T.corner[k], &T.corner[4 + k]);
-    } else if (t < 2 * NN + 9) {
-      const int k = t - 2 * NN - 4;
-      T.ct[k] = cospif(fmaf(0.25f * (float)k, X.dtT, X.tT));
+    for (int t = g.t; t < 2 * NN + 9; t += 32 * G) {
+      const int c = t - 2 * NN;                              // corner, then stage-time index
+      const bool y = t < 2 * NN ? t >= NN : c >= 2;
+      const float h = y ? V.hy : V.hx, z0 = y ? V.y0 : V.x0;
+      float z = c < 0 ? fmaf(h, xi[y ? t - NN : t], z0) : z0 + ((c & 1) ? h : 0.0f);
+      if (c >= 4) z = fmaf(0.25f * (float)(c - 4), X.f.dtT, X.f.tT);
+      float sn, cs;
+      sincospif(z, &sn, &cs);
+      if (c < 0) {
+        T.n[y ? 2 : 0][y ? t - NN : t] = sn;
+        T.n[y ? 3 : 1][y ? t - NN : t] = cs;
+      } else if (c < 4) {
+        T.corner[c] = sn;
+        T.corner[4 + c] = cs;
+      } else {
+        T.ct[c - 4] = cs;
+      }
     }
-  } else if (t < 5) {
-    T.ct[t] = 1.0f;
+  } else if (g.t < 5) {
+    T.ct[g.t] = 1.0f;
   }
 }
 
 // ------------------------------------------------------------------ phase 1
 template <int NN>
 struct Smem1 {
-  static constexpr int ND = Shape<NN>::ND, NP = Shape<NN>::NP, RS = Shape<NN>::RS, G = Shape<NN>::G;
+  static constexpr int ND = Shape<NN>::ND, NP = Shape<NN>::NP, RP = Shape<NN>::RP, G = Shape<NN>::G;
   __align__(16) float ph[NN * NP];             // psihat rows
   __align__(16) float psi[NN * NP];            // psi^n rows
   union {
     struct {                                   // the collocation solve
-      float r[ND], tt[ND], best[ND];
-      float Rx[NN * RS], Ry[NN * RS];
+      __align__(16) float r[NN * NP], tt[NN * RP], Rx[NN * RP], Ry[NN * RP];   // residual rows, columns of the row pass
+      float best[ND];
     } sv;
     struct {                                   // the face outflow, after the solve
-      float fbo[4][NMAX][3], fbi[4][NMAX][3];  // per face point and distinct stage: outflow, inflow weight
+      float fbo[4][NMAX][3];                   // per face point and distinct stage: outflow weight
       float fv[4][NMAX][3];                    //   and the outflow value (phi - r0)
       float pt[4][NMAX][4];                    // per face point: U_out, U_in, P1, P2 over the step
       float fs[4][4];                          // per face: the same summed over its points
       int items[4 * NMAX * 2];                 // outflow (point, stage) pairs that need a foot
     } fc;
   } u;
-  float red[4 * G];
+  float red[8 * G];
+  float trp[4 * NN];                           // traces of psi^n at the own face points
   int cum[5];
   int nitems;
   Trig<NN> T;
+  Elem el[2];                                  // this and the next element, its problem's record
+  const ProbGeom* geo[2];
   float sth[2][ND], stl[2][ND];                // staged input state (hi, lo) of this and the next element
 };
 
@@ -655,7 +773,7 @@ __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB)
     k_p1(StepParams P0, const __grid_constant__ Mixed2DExtra X0, Map2D M, int64_t count, const float* __restrict__ in,
          Work2M W, unsigned* status) {
   using S = Shape<NN>;
-  constexpr int ND = S::ND, NP = S::NP, RS = S::RS, G = S::G, GT = S::GT, EPC = S::EPC;
+  constexpr int ND = S::ND, NP = S::NP, RP = S::RP, G = S::G, GT = S::GT, EPC = S::EPC;
   __shared__ float s_xi[NN], s_lam[NN], s_w[NN], s_l0[NN], s_l1[NN];
   __shared__ Smem1<NN> sm_all[EPC];
   if (threadIdx.x < NN) {
@@ -678,14 +796,22 @@ __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB)
   const int p0 = t, p1 = t + GT;
   const bool v0 = p0 < ND, v1 = p1 < ND;
   const int i0 = p0 % NN, j0 = (p0 / NN) % NN, i1 = p1 % NN, j1 = (p1 / NN) % NN;
+  // w (x) w at the thread's nodes as float-float
+  const float2 w2h = make_float2(v0 ? X0.w2h[p0] : 0.0f, v1 ? X0.w2h[p1] : 0.0f);
+  const float2 w2l = make_float2(v0 ? X0.w2l[p0] : 0.0f, v1 ? X0.w2l[p1] : 0.0f);
   unsigned long long c_it = 0, c_floor = 0, c_nc = 0, c_feet = 0;
   unsigned bits = 0;
   const int64_t ngroups = (int64_t)gridDim.x * EPC;
-  // asynchronous copies of element kk's input state into staging buffer b (one group per call)
+  // asynchronous copies of element kk's input state into staging buffer b (one group per call); the element
+  // is resolved here, one iteration ahead
   auto stage = [&](int64_t kk, int b) {
     if (kk < count) {
-      StepParams Pn = P0;
-      const Elem En = elem_at<NN>(Pn, M, kk);
+      const ProbGeom* gn;
+      const Elem En = elem_at<NN>(P0, M, kk, gn);
+      if (t == 0) {
+        sm.el[b] = En;
+        sm.geo[b] = gn;
+      }
       if (v0) { cp_async4(&sm.sth[b][p0], in + En.base + p0); cp_async4(&sm.stl[b][p0], in + X0.plane + En.base + p0); }
       if (v1) { cp_async4(&sm.sth[b][p1], in + En.base + p1); cp_async4(&sm.stl[b][p1], in + X0.plane + En.base + p1); }
     }
@@ -695,15 +821,15 @@ __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB)
   stage(k, 0);
   for (int b = 0; k < count; k += ngroups, b ^= 1) {
     g.sync();                                    // the previous element's shared data is consumed
+    const Elem E = sm.el[b];
+    StepParams P = P0;
+    Mixed2DExtra X = X0;
+    use_problem(sm.geo[b], P, X);
     stage(k + ngroups, b ^ 1);
     cp_async_wait1();
-    StepParams P = P0;
-    const Elem E = elem_at<NN>(P, M, k);
-    Mixed2DExtra X = X0;
-    batch_extra(P, M, X);
     const int ex = E.ex, ey = E.ey;
-    const float x0 = (float)(P.x0 + ex * P.hx), y0 = (float)(P.y0 + ey * P.hy);
-    const VelElem V = make_vel(P, X, x0, y0);
+    const VelElem V = make_vel(P, X, corner_of(X.f.x0, X.f.x0l, X.f.hx, X.f.hxl, ex),
+                               corner_of(X.f.y0, X.f.y0l, X.f.hy, X.f.hyl, ey));
     trig_setup<NN>(g, V, X, s_xi, sm.T);
     g.sync();                                    // this element's staged state is visible
     const float* sh = sm.sth[b];
@@ -717,28 +843,22 @@ __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB)
       gy = ((c10 + c11) - (c00 + c01)) * X.span;
     }
     // psi^n at the own nodes, and the element mass in float-float
-    float pn0 = 0.0f, pn1 = 0.0f;
-    ff mn = {0.0f, 0.0f};
-    if (v0) {
-      const float hi = sh[p0], lo = sl[p0];
-      const ff L = lref(r0, gx, gy, s_xi[i0] - 0.5f, s_xi[j0] - 0.5f);
-      pn0 = __fadd_rn(__fsub_rn(hi, L.hi), __fsub_rn(lo, L.lo));
-      sm.psi[j0 * NP + i0] = pn0;
-      mn = ff_mul(ff{hi, lo}, ff{X.w2h[p0], X.w2l[p0]});
-    }
-    if (v1) {
-      const float hi = sh[p1], lo = sl[p1];
-      const ff L = lref(r0, gx, gy, s_xi[i1] - 0.5f, s_xi[j1] - 0.5f);
-      pn1 = __fadd_rn(__fsub_rn(hi, L.hi), __fsub_rn(lo, L.lo));
-      sm.psi[j1 * NP + i1] = pn1;
-      mn = ff_add(mn, ff_mul(ff{hi, lo}, ff{X.w2h[p1], X.w2l[p1]}));
-    }
+    const float2 hi2 = make_float2(v0 ? sh[p0] : 0.0f, v1 ? sh[p1] : 0.0f);
+    const float2 lo2 = make_float2(v0 ? sl[p0] : 0.0f, v1 ? sl[p1] : 0.0f);
+    const float2 ha = make_float2(s_xi[i0] - 0.5f, s_xi[i1] - 0.5f), hb = make_float2(s_xi[j0] - 0.5f, s_xi[j1] - 0.5f);
+    const ff2 L2 = lref2(r0, gx, gy, ha, hb);
+    const float2 pn2 = add2(sub2(hi2, L2.hi), sub2(lo2, L2.lo));
+    const float pn0 = v0 ? pn2.x : 0.0f, pn1 = v1 ? pn2.y : 0.0f;
+    if (v0) sm.psi[j0 * NP + i0] = pn0;
+    if (v1) sm.psi[j1 * NP + i1] = pn1;
+    const ff2 mn2 = ff_mul2(ff2{hi2, lo2}, w2h, w2l);
+    const ff mn = ff_add(ff{mn2.hi.x, mn2.lo.x}, ff{mn2.hi.y, mn2.lo.y});
     g.sync();
     // advect the particles of nodes p0, p1 in reference coordinates
     float2 d2x = bc2(0.0f), d2y = bc2(0.0f);
     rk_disp2(V, P.rk, make_float2(s_xi[i0], s_xi[i1]), make_float2(s_xi[j0], s_xi[j1]),
              make_float2(sm.T.n[0][i0], sm.T.n[0][i1]), make_float2(sm.T.n[1][i0], sm.T.n[1][i1]),
-             make_float2(sm.T.n[2][j0], sm.T.n[2][j1]), make_float2(sm.T.n[3][j0], sm.T.n[3][j1]), d2x, d2y, X.dt,
+             make_float2(sm.T.n[2][j0], sm.T.n[2][j1]), make_float2(sm.T.n[3][j0], sm.T.n[3][j1]), d2x, d2y, X.f.dt,
              sm.T.ct);
     const float dx0 = v0 ? d2x.x : 0.0f, dy0 = v0 ? d2y.x : 0.0f, dx1 = v1 ? d2x.y : 0.0f, dy1 = v1 ? d2y.y : 0.0f;
     float2 Lx[NN], Ly[NN];
@@ -747,51 +867,37 @@ __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB)
     // collocation data of psihat = phihat - L
     const float ps0 = v0 ? pn0 - fmaf(gx, dx0, gy * dy0) : 0.0f;
     const float ps1 = v1 ? pn1 - fmaf(gx, dx1, gy * dy1) : 0.0f;
-    const float2 md = g.sum2(dx0 + dx1, dy0 + dy1);
-    const float mdx = md.x / ND, mdy = md.y / ND;
+    float sdx = dx0 + dx1, sdy = dy0 + dy1, unused = 0.0f, scale = fmaxf(fabsf(ps0), fabsf(ps1));
+    g.sum3max(sdx, sdy, unused, scale, false);
+    const float mdx = sdx / ND, mdy = sdy / ND;
     // preconditioner: interpolation back over the mean displacement, Rx[i][q] = l_q(xi_i - mdx)
     if (t < 2 * NN) {
       float b[NN];
       const int row = t < NN ? t : t - NN;
       basis_at<NN>(s_xi, s_lam, s_xi[row], t < NN ? -mdx : -mdy, b);
-      float* R = (t < NN ? sm.u.sv.Rx : sm.u.sv.Ry) + row * RS;
+      float* R = (t < NN ? sm.u.sv.Rx : sm.u.sv.Ry) + row * RP;
 #pragma unroll
       for (int q = 0; q < NN; ++q) R[q] = b[q];
     }
-    if (v0) sm.u.sv.r[p0] = ps0;
-    if (v1) sm.u.sv.r[p1] = ps1;
+    if (v0) sm.u.sv.r[j0 * NP + i0] = ps0;
+    if (v1) sm.u.sv.r[j1 * NP + i1] = ps1;
     g.sync();
-    // psihat (+)= Ry r Rx^T
+    // psihat (+)= Ry r Rx^T: the row pass leaves its result by columns, so that both passes read rows
     auto precond = [&](bool first) {
-      if (v0) {
-        float acc = 0.0f;
-#pragma unroll
-        for (int q = 0; q < NN; ++q) acc = fmaf(sm.u.sv.Rx[i0 * RS + q], sm.u.sv.r[j0 * NN + q], acc);
-        sm.u.sv.tt[p0] = acc;
-      }
-      if (v1) {
-        float acc = 0.0f;
-#pragma unroll
-        for (int q = 0; q < NN; ++q) acc = fmaf(sm.u.sv.Rx[i1 * RS + q], sm.u.sv.r[j1 * NN + q], acc);
-        sm.u.sv.tt[p1] = acc;
-      }
+      if (v0) sm.u.sv.tt[i0 * RP + j0] = dot_rows<NN>(sm.u.sv.Rx + i0 * RP, sm.u.sv.r + j0 * NP);
+      if (v1) sm.u.sv.tt[i1 * RP + j1] = dot_rows<NN>(sm.u.sv.Rx + i1 * RP, sm.u.sv.r + j1 * NP);
       g.sync();
       if (v0) {
-        float acc = 0.0f;
-#pragma unroll
-        for (int q = 0; q < NN; ++q) acc = fmaf(sm.u.sv.Ry[j0 * RS + q], sm.u.sv.tt[q * NN + i0], acc);
+        const float acc = dot_rows<NN>(sm.u.sv.Ry + j0 * RP, sm.u.sv.tt + i0 * RP);
         sm.ph[j0 * NP + i0] = first ? acc : sm.ph[j0 * NP + i0] + acc;
       }
       if (v1) {
-        float acc = 0.0f;
-#pragma unroll
-        for (int q = 0; q < NN; ++q) acc = fmaf(sm.u.sv.Ry[j1 * RS + q], sm.u.sv.tt[q * NN + i1], acc);
+        const float acc = dot_rows<NN>(sm.u.sv.Ry + j1 * RP, sm.u.sv.tt + i1 * RP);
         sm.ph[j1 * NP + i1] = first ? acc : sm.ph[j1 * NP + i1] + acc;
       }
       g.sync();
     };
     precond(true);
-    const float scale = g.max(fmaxf(fabsf(ps0), fabsf(ps1)));
     // iterate to the tolerance; a residual that stalls at the float floor is accepted; the best
     // iterate is kept against divergence, and accepting it above the floor is reported
     float prev = INFINITY, best = INFINITY, rmax = INFINITY;
@@ -817,8 +923,8 @@ __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB)
         if (v1) sm.u.sv.best[p1] = sm.ph[j1 * NP + i1];
       }
       prev = rmax;
-      if (v0) sm.u.sv.r[p0] = r0v;
-      if (v1) sm.u.sv.r[p1] = r1v;
+      if (v0) sm.u.sv.r[j0 * NP + i0] = r0v;
+      if (v1) sm.u.sv.r[j1 * NP + i1] = r1v;
       g.sync();
       precond(false);
     }
@@ -846,36 +952,44 @@ __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB)
     if (v1) W.psihat[E.base + p1] = sm.ph[j1 * NP + i1];
     // element sums of psi^n (reference measure) and the float-float element mass
     const float w20 = v0 ? s_w[i0] * s_w[j0] : 0.0f, w21 = v1 ? s_w[i1] * s_w[j1] : 0.0f;
-    const float2 m12 = g.sum2(fmaf(w20, pn0, w21 * pn1), fmaf(w20 * pn0, pn0, w21 * pn1 * pn1));
-    const ff Mn = g.ffsum(mn);
+    float m1 = fmaf(w20, pn0, w21 * pn1), m2 = fmaf(w20 * pn0, pn0, w21 * pn1 * pn1);
+    const ff Mn = g.ffsum_sum2(mn, m1, m2);
     float* el = W.elem + E.g * 8;
     if (t == 0) {
       el[0] = r0;
       el[1] = gx;
       el[2] = gy;
-      el[3] = m12.x;
-      el[4] = m12.y;
+      el[3] = m1;
+      el[4] = m2;
       el[5] = Mn.hi;
       el[6] = Mn.lo;
     }
     // interface values at the face points (relative to L): traces of psihat, or phi^n at the
     // backward characteristic foot of the face point from t^{n+1} (eq. 4.11; meshes of one node
     // count), L(foot) - L(face point) being the linear part over the foot's displacement
+    float ub = 0.0f, tr0 = 0.0f;                 // own face point: u.n at ct = 1, the trace of psi^n
+    const bool flux = (P.cons & (SL_C_MASS | SL_C_ENERGY)) != 0;
+    static_assert(4 * NN <= GT, "a thread per own face point");
     if (t < 4 * NN) {
       const int f = t / NN, q = t % NN;
+      const float xr = f == 0 ? 0.0f : f == 1 ? 1.0f : s_xi[q];
+      const float yr = f == 2 ? 0.0f : f == 3 ? 1.0f : s_xi[q];
+      float Sx = 0.0f, Cx = 0.0f, Sy = 0.0f, Cy = 0.0f;
+      if (V.kind == SL_VEL_SWIRL && !V.direct) {
+        Sx = f < 2 ? sm.T.corner[f] : sm.T.n[0][q];
+        Cx = f < 2 ? sm.T.corner[4 + f] : sm.T.n[1][q];
+        Sy = f < 2 ? sm.T.n[2][q] : sm.T.corner[f];
+        Cy = f < 2 ? sm.T.n[3][q] : sm.T.corner[4 + f];
+      }
+      float ur, vr;
+      vel_base(V, xr, yr, Sx, Cx, Sy, Cy, 1.0f, ur, vr);
+      ub = (f == 0 || f == 2 ? -1.0f : 1.0f) * (f < 2 ? ur * X.f.hx : vr * X.f.hy);
+      const float* Lb = (f == 1 || f == 3) ? s_l1 : s_l0;
+      const int at = f < 2 ? q * NP : q, st = f < 2 ? 1 : NP;
       float acc = 0.0f;
       if (P.bvalue == SL_BV_BACKTRACK) {
-        const float xr = f == 0 ? 0.0f : f == 1 ? 1.0f : s_xi[q];
-        const float yr = f == 2 ? 0.0f : f == 3 ? 1.0f : s_xi[q];
-        float Sx = 0.0f, Cx = 0.0f, Sy = 0.0f, Cy = 0.0f;
-        if (V.kind == SL_VEL_SWIRL && !V.direct) {
-          Sx = f < 2 ? sm.T.corner[f] : sm.T.n[0][q];
-          Cx = f < 2 ? sm.T.corner[4 + f] : sm.T.n[1][q];
-          Sy = f < 2 ? sm.T.n[2][q] : sm.T.corner[f];
-          Cy = f < 2 ? sm.T.n[3][q] : sm.T.corner[4 + f];
-        }
         float fdx = 0.0f, fdy = 0.0f;
-        rk_disp(V, P.rk, xr, yr, Sx, Cx, Sy, Cy, fdx, fdy, -X.dt, 1.0f, -1.0f, sm.T.ct);
+        rk_disp(V, P.rk, xr, yr, Sx, Cx, Sy, Cy, fdx, fdy, -X.f.dt, 1.0f, -1.0f, sm.T.ct);
         float bx[NN], by[NN];
         basis_at<NN>(s_xi, s_lam, xr, fdx, bx);
         basis_at<NN>(s_xi, s_lam, yr, fdy, by);
@@ -883,11 +997,21 @@ __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB)
         for (int mm = 0; mm < NN; ++mm) acc = fmaf(by[mm], row_dot<NN>(sm.psi + mm * NP, bx), acc);
         acc += fmaf(gx, fdx, gy * fdy);
       } else {
-        const float* Lb = (f == 1 || f == 3) ? s_l1 : s_l0;
+        float a2 = 0.0f;
 #pragma unroll
-        for (int kk = 0; kk < NN; ++kk) acc = fmaf(f < 2 ? sm.ph[q * NP + kk] : sm.ph[kk * NP + q], Lb[kk], acc);
+        for (int kk = 0; kk < NN; ++kk) {
+          acc = fmaf(sm.ph[at + kk * st], Lb[kk], acc);
+          a2 = fmaf(sm.psi[at + kk * st], Lb[kk], a2);
+        }
+        tr0 = a2;
+        sm.trp[t] = a2;
       }
       W.traces[E.g * M.tstride + t] = acc;
+      // the upwind side of the face point at t^{n+1} (eq. 4.12a): 0 own, 1 the neighbour's or the ghost, 2 tie
+      if (P.cons & SL_C_BOUNDARY) {
+        const float un = ub * sm.T.ct[4];
+        W.side[E.g * M.tstride + t] = un > (float)TIE ? 0 : un < -(float)TIE ? 1 : 2;
+      }
     }
     // outflow over each face and step; a face shared with a neighbour of another node count takes
     // the rule of the finer side, so that both elements integrate the same points.  Pass 1 (one face
@@ -895,7 +1019,7 @@ __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB)
     // the stage time t^n the outflow value itself (the trace of psi^n, no foot).  Pass 2: the outflow
     // (point, stage) pairs of later stage times, compacted into a list, one backward characteristic
     // foot each.  Every pair writes its own slot; the face sums add the slots in a fixed order.
-    if (P.cons & (SL_C_MASS | SL_C_ENERGY)) {
+    if (flux) {
       if (t < 4) {
         // points of face t and their prefix sum (lanes 0-3 of the first warp)
         const int nb = nb_index(P, ex, ey, t);
@@ -918,8 +1042,8 @@ __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB)
       // Geometry of face point idx: face, point, rule, reference coordinates, sines and cosines.
       // CONF: every face takes the element's own rule (conforming neighbours), so that no lane
       // carries the general rule's branches.
-      auto face_point = [&](auto conf, int idx, int& f, int& q, int& nq, float& xr, float& yr, float& Sx, float& Cx,
-                            float& Sy, float& Cy) {
+      auto face_point = [&](auto conf, int idx, int& f, int& q, int& nq, float& zq, float& xr, float& yr, float& Sx,
+                            float& Cx, float& Sy, float& Cy) {
         constexpr bool CONF = decltype(conf)::value;
         if (CONF) {
           f = idx / NN;
@@ -930,7 +1054,7 @@ __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB)
           q = idx - sm.cum[f];
           nq = sm.cum[f + 1] - sm.cum[f];
         }
-        const float zq = (CONF || nq == NN) ? s_xi[q] : X.rules[(size_t)nq * 3 * NMAX + q];
+        zq = (CONF || nq == NN) ? s_xi[q] : X.rules[(size_t)nq * 3 * NMAX + q];
         xr = f == 0 ? 0.0f : f == 1 ? 1.0f : zq;
         yr = f == 2 ? 0.0f : f == 3 ? 1.0f : zq;
         Sx = Cx = Sy = Cy = 0.0f;
@@ -956,44 +1080,46 @@ __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB)
       constexpr bool TAB = decltype(tabc)::value;
       for (int idx = t; idx < total; idx += GT) {
         int f, q, nq;
-        float xr, yr, Sx, Cx, Sy, Cy;
-        face_point(conf, idx, f, q, nq, xr, yr, Sx, Cx, Sy, Cy);
-        const float hn = f < 2 ? X.hx : X.hy;            // velocity in reference units times this = u.n
+        float zq, xr, yr, Sx, Cx, Sy, Cy;
+        face_point(conf, idx, f, q, nq, zq, xr, yr, Sx, Cx, Sy, Cy);
+        const float hn = f < 2 ? X.f.hx : X.f.hy;            // velocity in reference units times this = u.n
         const float sg = (f == 0 || f == 2) ? -1.0f : 1.0f;
-        const float Wq = (f < 2 ? X.hy : X.hx) *
+        const float Wq = (f < 2 ? X.f.hy : X.f.hx) *
                          ((CONF || nq == NN) ? s_w[q] : X.rules[(size_t)nq * 3 * NMAX + 2 * NMAX + q]);
-        // phi - r0 at the face point itself (stage time t^n): the trace of psi^n plus (L - r0)
-        float val0;
-        if (CONF || nq == NN) {
+        // phi - r0 at the face point itself (stage time t^n): the trace of psi^n plus (L - r0); u.n at ct = 1
+        float val0, ubase;
+        if (CONF && P.bvalue != SL_BV_BACKTRACK) {
+          val0 = tr0;                              // this thread's own face point, formed with the traces
+        } else if (CONF || nq == NN) {
           const float* Lb = (f == 1 || f == 3) ? s_l1 : s_l0;
           float acc = 0.0f;
 #pragma unroll
           for (int kk = 0; kk < NN; ++kk) acc = fmaf(f < 2 ? sm.psi[q * NP + kk] : sm.psi[kk * NP + q], Lb[kk], acc);
           val0 = acc;
         } else {
-          float bx[NN], by[NN];
-          basis_at<NN>(s_xi, s_lam, xr, 0.0f, bx);
-          basis_at<NN>(s_xi, s_lam, yr, 0.0f, by);
+          // a point of another rule: the own traces interpolated along the face (with backtracked values the
+          // mesh has one node count)
+          float bt[NN];
+          basis_at<NN>(s_xi, s_lam, zq, 0.0f, bt);
           float acc = 0.0f;
 #pragma unroll
-          for (int mm = 0; mm < NN; ++mm) acc = fmaf(by[mm], row_dot<NN>(sm.psi + mm * NP, bx), acc);
+          for (int mm = 0; mm < NN; ++mm) acc = fmaf(bt[mm], sm.trp[f * NN + mm], acc);
           val0 = acc;
         }
         val0 += fmaf(gx, xr - 0.5f, gy * (yr - 0.5f));
+        if (CONF) {
+          ubase = ub;
+        } else {
+          float ur, vr;
+          vel_base(V, xr, yr, Sx, Cx, Sy, Cy, 1.0f, ur, vr);
+          ubase = sg * (f < 2 ? ur : vr) * hn;
+        }
         // per distinct stage time: the sign of u.n, the weight; later stage times that flow out
         // are queued for their backward foot (their weight kept in fbo, 0 otherwise)
         float uo = 0.0f, ui = 0.0f, q1 = 0.0f, q2 = 0.0f;
         for (int s = 0; s < S; ++s) {
           const float cs = c_ds_c[P.rk][s];
-          float ur, vr;
-          const float ct = sm.T.ct[__float2int_rn(4.0f * cs)];
-          if (TAB) {
-            ur = Sx * Sx * (2.0f * Sy * Cy) * ct * V.ihx;
-            vr = -Sy * Sy * (2.0f * Sx * Cx) * ct * V.ihy;
-          } else {
-            vel_at(V, xr, yr, Sx, Cx, Sy, Cy, 0.0f, 0.0f, ct, ur, vr);
-          }
-          const float un = sg * (f < 2 ? ur : vr) * hn;
+          const float un = ubase * sm.T.ct[__float2int_rn(4.0f * cs)];
           const float bw = c_ds_b[P.rk][s] * Wq * un;
           const bool out = un > (float)TIE;
           if (out) uo += bw;
@@ -1032,12 +1158,12 @@ __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB)
         const int code = sm.u.fc.items[it2];
         const int idx = code >> 2, s = code & 3;
         int f, q, nq;
-        float xr, yr, Sx, Cx, Sy, Cy;
-        if (conforming) face_point(std::true_type{}, idx, f, q, nq, xr, yr, Sx, Cx, Sy, Cy);
-        else face_point(std::false_type{}, idx, f, q, nq, xr, yr, Sx, Cx, Sy, Cy);
+        float zq, xr, yr, Sx, Cx, Sy, Cy;
+        if (conforming) face_point(std::true_type{}, idx, f, q, nq, zq, xr, yr, Sx, Cx, Sy, Cy);
+        else face_point(std::false_type{}, idx, f, q, nq, zq, xr, yr, Sx, Cx, Sy, Cy);
         const float cs = c_ds_c[P.rk][s];
         float fdx = 0.0f, fdy = 0.0f;
-        rk_disp(V, P.rk, xr, yr, Sx, Cx, Sy, Cy, fdx, fdy, -cs * X.dt, cs, -cs, sm.T.ct);
+        rk_disp(V, P.rk, xr, yr, Sx, Cx, Sy, Cy, fdx, fdy, -cs * X.f.dt, cs, -cs, sm.T.ct);
         float bx[NN], by[NN];
         basis_at<NN>(s_xi, s_lam, xr, fdx, bx);
         basis_at<NN>(s_xi, s_lam, yr, fdy, by);
@@ -1071,9 +1197,12 @@ __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB)
         const int f = t >> 2, c = t & 3;
         const int nq = sm.cum[f + 1] - sm.cum[f];
         float acc = 0.0f;
+        if (conforming) {
 #pragma unroll
-        for (int q = 0; q < NMAX; ++q)
-          if (q < nq) acc += sm.u.fc.pt[f][q][c];
+          for (int q = 0; q < NN; ++q) acc += sm.u.fc.pt[f][q][c];
+        } else {
+          for (int q = 0; q < nq; ++q) acc += sm.u.fc.pt[f][q][c];
+        }
         sm.u.fc.fs[f][c] = acc;
       }
       g.sync();
@@ -1104,13 +1233,21 @@ __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB)
 }
 
 // ------------------------------------------------------------------ phase 2
+// the neighbour's trace across a p-nonconforming face, out of line: its 2 x 17 products in registers would set
+// the register count of the whole kernel
+static __device__ __noinline__ float interp_far(const float* rules, int nn, const float* tr, float z) {
+  return interp_rule(rules, nn, tr, z);
+}
+
 template <int NN>
 struct Smem2 {
   static constexpr int ND = Shape<NN>::ND, G = Shape<NN>::G;
   static constexpr int MMAX = 4 * NN + 1;
+  __align__(16) float2 r[(MMAX + 1) & ~1];     // residuals, each twice (operands of the paired products)
+  __align__(16) float2 ca[(MMAX + 1) & ~1];
   float a[ND];
-  float r[MMAX], ca[MMAX];
-  float red[4 * G];
+  int rows[G];                                 // per warp: faces with a non-zero residual among its points
+  float red[8 * G];
   float scal[8];
 };
 
@@ -1122,15 +1259,19 @@ __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB2)
   constexpr int ND = S::ND, G = S::G, GT = S::GT, EPC = S::EPC;
   __shared__ float s_xi[NN], s_w[NN], s_l0[NN], s_l1[NN];
   __shared__ Smem2<NN> sm_all[EPC];
-  // the pseudo-inverse of the fit, [m][n^2], staged once per CTA (dynamic shared memory)
-  extern __shared__ __align__(16) float s_Cp[];
+  // the pseudo-inverse of the fit by row, a thread's two nodes side by side (zero where it has none), staged
+  // once per CTA (dynamic shared memory): one 8-byte load and one paired FMA per row and thread
+  extern __shared__ __align__(16) float2 s_Cp[];               // [m][GT]
   if (threadIdx.x < NN) {
     s_xi[threadIdx.x] = X0.xi[threadIdx.x];
     s_w[threadIdx.x] = X0.w[threadIdx.x];
     s_l0[threadIdx.x] = X0.l0[threadIdx.x];
     s_l1[threadIdx.x] = X0.l1[threadIdx.x];
   }
-  for (int i = threadIdx.x; i < P0.m * ND; i += blockDim.x) s_Cp[i] = X0.Cp[i];
+  for (int i = threadIdx.x; i < P0.m * GT; i += blockDim.x) {
+    const int kk = i / GT, c = i % GT;
+    s_Cp[i] = make_float2(c < ND ? X0.Cp[kk * ND + c] : 0.0f, c + GT < ND ? X0.Cp[kk * ND + c + GT] : 0.0f);
+  }
   __syncthreads();
   Grp<G> g;
   g.slot = threadIdx.x / GT;
@@ -1151,12 +1292,11 @@ __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB2)
   for (int64_t k = (int64_t)blockIdx.x * EPC + g.slot; k < count; k += ngroups) {
     g.sync();
     StepParams P = P0;
-    const Elem E = elem_at<NN>(P, M, k);
+    const ProbGeom* geo;
+    const Elem E = elem_at<NN>(P0, M, k, geo);
     Mixed2DExtra X = X0;
-    batch_extra(P, M, X);
+    use_problem(geo, P, X);
     const int ex = E.ex, ey = E.ey;
-    const float x0 = (float)(P.x0 + ex * P.hx), y0 = (float)(P.y0 + ey * P.hy);
-    const VelElem V = make_vel(P, X, x0, y0);
     // every global read of the element first, so that they share one memory round trip: own
     // record, psihat, input (energy), face-point traces and the neighbours' records and faces
     const bool bnd = (P.cons & SL_C_BOUNDARY) != 0;
@@ -1172,13 +1312,14 @@ __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB2)
       if (v1) { in_hi1 = in[E.base + p1]; in_lo1 = in[X.plane + E.base + p1]; }
     }
     // boundary lanes: face point (f, q), own trace, neighbour's trace at this point and record
-    int bf = 0, bq = 0, bnb = -1;
+    int bf = 0, bq = 0, bnb = -1, bside = 0;
     float own = 0.0f, trn = 0.0f, en0 = 0.0f, en1 = 0.0f, en2 = 0.0f;
     if (bnd && t < 4 * NN) {
       bf = t / NN;
       bq = t % NN;
       bnb = nb_index(P, ex, ey, bf);
       own = W.traces[E.g * M.tstride + t];
+      bside = W.side[E.g * M.tstride + t];
       if (bnb >= 0) {
         const int64_t gn = E.gb + bnb;
         const int nn = order_of<NN>(M, gn);
@@ -1187,7 +1328,7 @@ __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB2)
         en0 = en[0];
         en1 = en[1];
         en2 = en[2];
-        trn = nn == NN ? tr[bq] : interp_rule(X.rules, nn, tr, s_xi[bq]);
+        trn = nn == NN ? tr[bq] : interp_far(X.rules, nn, tr, s_xi[bq]);
       }
     }
     // face lanes (0-3): own face record, the neighbour's record of the shared face and its r0
@@ -1205,6 +1346,7 @@ __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB2)
         rnb = W.elem[(E.gb + fnb) * 8];
       }
     }
+    float rr = 0.0f;
     if (bnd && t < 4 * NN) {
       const int f = bf, q = bq, nb = bnb;
       // neighbour's value at this element's face point relative to this element's L: the difference
@@ -1221,18 +1363,9 @@ __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB2)
       } else {
         other = __fsub_rn(__fsub_rn((float)P.ghost, lown.hi), lown.lo);
       }
-      const float xr = f == 0 ? 0.0f : f == 1 ? 1.0f : s_xi[q];
-      const float yr = f == 2 ? 0.0f : f == 3 ? 1.0f : s_xi[q];
-      // one velocity evaluation per face point at t^{n+1}: sinpi/cospi directly
-      VelElem Vd = V;
-      Vd.direct = true;
-      const float ct = V.kind == SL_VEL_SWIRL ? cospif(X.tT + X.dtT) : 1.0f;
-      float ur, vr;
-      vel_at(Vd, xr, yr, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, ct, ur, vr);
-      const float un = (f == 0 || f == 2 ? -1.0f : 1.0f) * (f < 2 ? ur * X.hx : vr * X.hy);
       float val;
-      if (un > (float)TIE) val = own;
-      else if (un < -(float)TIE) val = other;
+      if (bside == 0) val = own;
+      else if (bside == 1) val = other;
       else val = nb < 0 ? own : 0.5f * (own + other);
       // the row's value at psihat: the own trace when the interface values are traces of psihat,
       // else the trace formed here from the stored psihat
@@ -1244,7 +1377,23 @@ __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB2)
 #pragma unroll
         for (int kk = 0; kk < NN; ++kk) trh = fmaf(f < 2 ? ps[q * NN + kk] : ps[kk * NN + q], Lb[kk], trh);
       }
-      sm.r[t] = val - trh;
+      rr = val - trh;
+      sm.r[t] = bc2(rr);
+    }
+    // faces whose rows all vanish (outflow faces: the own trace) add nothing to the fit
+    if (bnd && 32 * g.w < 4 * NN) {
+      const unsigned nz = __ballot_sync(0xffffffffu, !(rr == 0.0f));
+      int rows = 0;
+#pragma unroll
+      for (int f = 0; f < 4; ++f) {
+        const int lo = f * NN - 32 * g.w, hi = lo + NN;        // lanes of face f in this warp
+        const unsigned a = lo <= 0 ? 0xffffffffu : lo >= 32 ? 0u : 0xffffffffu << lo;
+        const unsigned b = hi >= 32 ? 0xffffffffu : hi <= 0 ? 0u : (1u << hi) - 1u;
+        rows |= (nz & a & b) ? 1 << f : 0;
+      }
+      if (g.lane == 0) sm.rows[g.w] = rows;
+    } else if (g.lane == 0) {
+      sm.rows[g.w] = 0;
     }
     // net outflow of mass (increments), of the squared increments and of the velocity, lanes 0-3 of
     // the first warp one face each, summed in face order; the float-float mass target
@@ -1277,7 +1426,7 @@ __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB2)
       }
       if (t == 0) {
         // M^{n+1} = M^n - dt / (hx hy) (net outflow), in float-float
-        const ff ln = ff_mul(sn, ff{X.lam_hi, X.lam_lo});
+        const ff ln = ff_mul(sn, ff{X.f.lam_hi, X.f.lam_lo});
         const ff target = ff_add(ff{mn_hi, mn_lo}, ff_neg(ln));
         sm.scal[0] = smm;
         sm.scal[1] = sd;
@@ -1289,26 +1438,30 @@ __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB2)
     g.sync();
     const float netm = sm.scal[0], netd2 = sm.scal[1];
     const ff target = {sm.scal[3], sm.scal[4]};
-    const float lam = X.dt_area;                  // dt / (hx hy)
+    const float lam = X.f.lam_hi;                 // dt / (hx hy)
     if (mass) {
       const float mh = g.sum(fmaf(w20, ph0, w21 * ph1));
       // target (increments): sum w psi^n - lam (net increment outflow + ref * closed-surface u.n);
       // ref * (closed-surface integral of u.n) is dropped: every 2D velocity here is divergence free
       // and the face quadrature integrates it to rounding (the refinement below meets the float-float
       // target whatever this residual leaves)
-      if (t == 0) sm.r[nb_rows] = (m1 - lam * netm) - mh;
+      if (t == 0) sm.r[nb_rows] = bc2((m1 - lam * netm) - mh);
     }
     g.sync();
     const int m = P.m;
-    float phL0 = ph0, phL1 = ph1;
-#pragma unroll 4
-    for (int kk = 0; kk < m; ++kk) {
-      const float rk_ = sm.r[kk];
-      phL0 = fmaf(s_Cp[kk * ND + (v0 ? p0 : 0)], rk_, phL0);
-      phL1 = fmaf(s_Cp[kk * ND + (v1 ? p1 : 0)], rk_, phL1);
-    }
-    if (!v0) phL0 = 0.0f;
-    if (!v1) phL1 = 0.0f;
+    float2 L2 = make_float2(ph0, ph1);
+    int rows = 0;
+#pragma unroll
+    for (int w = 0; w < G; ++w) rows |= sm.rows[w];
+#pragma unroll
+    for (int f = 0; f < 4; ++f)
+      if (rows & (1 << f)) {
+        const float2* c = s_Cp + f * NN * GT + t;
+#pragma unroll
+        for (int kk = 0; kk < NN; ++kk) L2 = fma2(c[kk * GT], sm.r[f * NN + kk], L2);
+      }
+    if (mass) L2 = fma2(s_Cp[nb_rows * GT + t], sm.r[nb_rows], L2);
+    const float phL0 = L2.x, phL1 = L2.y;
     float cur0 = phL0, cur1 = phL1;
     bool ok = true;
     if (energy) {
@@ -1324,14 +1477,14 @@ __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB2)
         psin1 = __fadd_rn(__fsub_rn(in_hi1, L.hi), __fsub_rn(in_lo1, L.lo));
       }
       const float dp0 = phL0 - psin0, dp1 = phL1 - psin1;
-      const float2 evml = g.sum2(fmaf(w20 * dp0, phL0 + (phL0 - dp0), w21 * dp1 * (phL1 + (phL1 - dp1))),
-                                 fmaf(w20, phL0, w21 * phL1));
-      const float ev = evml.x, ml = evml.y;
+      float ev = fmaf(w20 * dp0, phL0 + (phL0 - dp0), w21 * dp1 * (phL1 + (phL1 - dp1)));
+      float ml = fmaf(w20, phL0, w21 * phL1);
+      float escale = fmaf(w20 * (r0 + cur0), r0 + cur0, w21 * (r0 + cur1) * (r0 + cur1));
+      float smax = fmaxf(fmaxf(fabsf(phL0), fabsf(phL1)), fabsf(r0));
+      g.sum3max(ev, ml, escale, smax, true);
       float gamma;
       if (mass) gamma = ev + lam * netd2;
       else gamma = fmaf(2.0f * r0, (ml - m1) + lam * netm, ev + lam * netd2);
-      const float escale = g.sum(fmaf(w20 * (r0 + cur0), r0 + cur0, w21 * (r0 + cur1) * (r0 + cur1)));
-      const float smax = g.max(fmaxf(fmaxf(fabsf(phL0), fabsf(phL1)), fabsf(r0)));
       if (smax >= 1e-30f && fabsf(gamma) > (float)ENERGY_SKIP_RTOL_MIXED * escale) {
         ++c_eapp;
         int exn;
@@ -1353,22 +1506,17 @@ __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB2)
             const float* Lb = (f == 1 || f == 3) ? s_l1 : s_l0;
             float acc = 0.0f;
             for (int kk = 0; kk < NN; ++kk) acc = fmaf(f < 2 ? sm.a[qq * NN + kk] : sm.a[kk * NN + qq], Lb[kk], acc);
-            sm.ca[t] = acc;
+            sm.ca[t] = bc2(-acc);
           }
           if (mass) {
             const float cmm = g.sum(fmaf(w20, a0, w21 * a1));
-            if (t == 0) sm.ca[nb_rows] = cmm;
+            if (t == 0) sm.ca[nb_rows] = bc2(-cmm);
           }
           g.sync();
-          float q0 = a0, q1 = a1;
+          float2 q2 = make_float2(a0, a1);
 #pragma unroll 4
-          for (int kk = 0; kk < m; ++kk) {
-            const float ck = sm.ca[kk];
-            q0 = fmaf(-s_Cp[kk * ND + (v0 ? p0 : 0)], ck, q0);
-            q1 = fmaf(-s_Cp[kk * ND + (v1 ? p1 : 0)], ck, q1);
-          }
-          if (!v0) q0 = 0.0f;
-          if (!v1) q1 = 0.0f;
+          for (int kk = 0; kk < m; ++kk) q2 = fma2(s_Cp[kk * GT + t], sm.ca[kk], q2);
+          const float q0 = q2.x, q1 = q2.y;
           const float2 ab = g.sum2(fmaf(w20 * ql0, q0, w21 * ql1 * q1), fmaf(w20 * q0, q0, w21 * q1 * q1));
           float alpha = ab.x;
           if (!mass) alpha = fmaf(rf, g.sum(fmaf(w20, q0, w21 * q1)), alpha);
@@ -1418,9 +1566,9 @@ __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB2)
       if (v1) mv = ff_add(mv, ff_mul(vv1, ff{X.w2h[p1], X.w2l[p1]}));
       mv = g.ffsum(mv);
       const float miss = ff_to_f(ff_add(target, ff_neg(mv)));
-      const float* cmcol = s_Cp + nb_rows * ND;
-      if (v0) vv0 = fast_two_sum(vv0.hi, fmaf(miss, cmcol[p0], vv0.lo));
-      if (v1) vv1 = fast_two_sum(vv1.hi, fmaf(miss, cmcol[p1], vv1.lo));
+      const float2 cm = s_Cp[nb_rows * GT + t];
+      if (v0) vv0 = fast_two_sum(vv0.hi, fmaf(miss, cm.x, vv0.lo));
+      if (v1) vv1 = fast_two_sum(vv1.hi, fmaf(miss, cm.y, vv1.lo));
     }
     if (v0) {
       out[E.base + p0] = vv0.hi;
@@ -1455,7 +1603,7 @@ void launch_n(int phase, const StepParams& p, const Mixed2DExtra& x, const Map2D
   using S = Shape<NN>;
   // phase 2 stages the fit operator for the largest row set (4 n + 1 rows), whatever p.m is, so
   // that one occupancy figure serves every launch
-  const size_t smem2 = (size_t)(4 * NN + 1) * S::ND * sizeof(float);
+  const size_t smem2 = (size_t)(4 * NN + 1) * S::GT * sizeof(float2);
   const void* kern = phase == 1 ? (const void*)k_p1<NN> : (const void*)k_p2<NN>;
   int fill = persistent_grid(kern, S::NT, phase == 1 ? 0 : smem2);
   // per_sm > 0: that many resident CTAs per SM (the autotuner's choice), within the occupancy

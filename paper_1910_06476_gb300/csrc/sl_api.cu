@@ -193,6 +193,27 @@ void build_rules(int basis, TableBufs& B, size_t& off, size_t& foff) {
 namespace sl {
 void set_global_error(const std::string& msg) { g_init_err = msg; }
 
+GeoF make_geof(double x0, double y0, double hx, double hy, double t, double dt, double Tper) {
+  GeoF f{};
+  auto two = [](double v, float& hi, float& lo) {
+    hi = (float)v;
+    lo = (float)(v - (double)hi);
+  };
+  two(x0, f.x0, f.x0l);
+  two(y0, f.y0, f.y0l);
+  two(hx, f.hx, f.hxl);
+  two(hy, f.hy, f.hyl);
+  f.ihx = (float)(1.0 / hx);
+  f.ihy = (float)(1.0 / hy);
+  f.dt = (float)dt;
+  two(dt / (hx * hy), f.lam_hi, f.lam_lo);
+  if (Tper != 0.0) {
+    f.tT = (float)(t / Tper);
+    f.dtT = (float)(dt / Tper);
+  }
+  return f;
+}
+
 int sm_count() {
   static std::mutex mu;
   static std::map<int, int> cache;
@@ -314,7 +335,7 @@ sl_status finish_uniform(sl_ctx* c) {
   alias_ntab(c);
   const size_t work_bytes = M.dim != 2 ? 0
                             : c->precision == SL_FP64 ? work2d_doubles(c->nvals, c->nel, 4 * c->n) * sizeof(double)
-                                                      : work2m_floats(c->nel, c->n) * sizeof(float);
+                                                      : work2m_floats(c->nvals, c->nel, 4 * c->n) * sizeof(float);
   return alloc_upload(c, B, work_bytes);
 }
 
@@ -347,7 +368,7 @@ sl_status finish_mapped(sl_ctx* c, const std::vector<uint16_t>& prob = {}) {
   }
   const size_t work_bytes = c->precision == SL_FP64
                                 ? (size_t)work2d_doubles(c->nvals, nel, 4 * NMAX) * sizeof(double)
-                                : (size_t)(c->nvals + nel * (4 * NMAX + WORK2M_FACE + WORK2M_ELEM)) * sizeof(float);
+                                : (size_t)work2m_floats(c->nvals, nel, 4 * NMAX) * sizeof(float);
   sl_status st = alloc_upload(c, B, work_bytes);
   if (st != SL_OK) return st;
   const bool batch = !prob.empty();
@@ -662,27 +683,15 @@ sl_status step2d_general(sl_ctx* c, StepParams P, const sl_velocity* vel, double
         X.linref = (opt->constraints & SL_C_ENERGY) ? 0 : 1;
         X.plane = plane_stride(c->nvals);
         X.span = (float)(0.5 / (N.b.xi[n - 1] - N.b.xi[0]));
-        X.hx = (float)hx;
-        X.hy = (float)hy;
-        X.ihx = (float)(1.0 / hx);
-        X.ihy = (float)(1.0 / hy);
+        X.f = make_geof(M.x0, M.y0, hx, hy, t, dt, vel->kind == SL_VEL_SWIRL ? vel->p[0] : 0.0);
         X.a = (float)vel->p[0];
         X.b = (float)vel->p[1];
         X.om = (float)vel->p[0];
         X.cx = (float)vel->p[1];
         X.cy = (float)vel->p[2];
-        X.dt = (float)dt;
-        const double lam = dt / (hx * hy);
-        X.dt_area = (float)lam;
-        X.lam_hi = (float)lam;
-        X.lam_lo = (float)(lam - (double)X.lam_hi);
-        if (vel->kind == SL_VEL_SWIRL) {
-          X.tT = (float)(t / vel->p[0]);
-          X.dtT = (float)(dt / vel->p[0]);
-          X.Tper = vel->p[0];
-        }
         float* W = (float*)c->d_work;
-        Work2M w{W, W + c->nvals, W + c->nvals + nel * ts, W + c->nvals + nel * (ts + WORK2M_FACE)};
+        Work2M w{W, W + c->nvals, W + c->nvals + nel * ts, W + c->nvals + nel * (ts + WORK2M_FACE),
+               (uint8_t*)(W + c->nvals + nel * (ts + WORK2M_FACE + WORK2M_ELEM))};
         launch_step2d_mixed(phase, n, P, X, map, count, (const float*)in, (float*)out, w, c->d_status, c->stream,
                             c->k2m_per_sm[phase - 1]);
         SL_CUDA(c, cudaGetLastError());
@@ -822,13 +831,19 @@ sl_status step_dispatch(sl_ctx* c, const void* phi_in, void* phi_out, const sl_v
   return SL_OK;
 }
 
+// time and step of one problem of a batch
+void set_geo_step(ProbGeom& G, const sl_velocity* vel, double t, double dt) {
+  G.t = t;
+  G.dt = dt;
+  G.f = make_geof(G.x0, G.y0, G.hx, G.hy, t, dt, vel->kind == SL_VEL_SWIRL ? vel->p[0] : 0.0);
+}
+
 // per-problem times and steps of a batch into its device geometry table
 sl_status set_batch_steps(sl_ctx* c, const sl_velocity* vel, const double* t, const double* dt) {
   for (int p = 0; p < c->nprob; ++p) {
     sl_status st = check_dt(c, c->prob_mesh[p], vel, t[p], dt[p]);
     if (st != SL_OK) return st;
-    c->geo_host[p].t = t[p];
-    c->geo_host[p].dt = dt[p];
+    set_geo_step(c->geo_host[p], vel, t[p], dt[p]);
   }
   SL_CUDA(c, cudaMemcpyAsync(c->d_geo, c->geo_host.data(), c->geo_host.size() * sizeof(ProbGeom),
                              cudaMemcpyHostToDevice, c->stream));
@@ -929,8 +944,7 @@ sl_status sl_run(sl_ctx* c, void* phi_a, void* phi_b, const sl_velocity* vel, do
       for (int s = 0; s < nsteps; ++s)
         for (int p = 0; p < c->nprob; ++p) {
           g[(size_t)s * c->nprob + p] = c->geo_host[p];
-          g[(size_t)s * c->nprob + p].t = t0 + s * dt;
-          g[(size_t)s * c->nprob + p].dt = dt;
+          set_geo_step(g[(size_t)s * c->nprob + p], vel, t0 + s * dt, dt);
         }
       SL_CUDA(c, cudaMemcpy(c->d_geo_run, g.data(), need * sizeof(ProbGeom), cudaMemcpyHostToDevice));
     }

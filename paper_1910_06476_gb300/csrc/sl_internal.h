@@ -111,6 +111,15 @@ void build_shift1d(const Basis1D& B, double a, double dt, double h, int rk, Shif
 void launch_step1d_f64(int n, const StepParams& p, const Tables1D& tb, const Shift1D* h, const double* xi_host,
                        const double* in, double* out, unsigned* status, cudaStream_t s);
 
+// Float parameters of one problem's geometry and step for the mixed 2D kernels, formed in double on the host;
+// pairs (x, xl) are float-float values
+struct GeoF {
+  float x0, x0l, y0, y0l, hx, hxl, hy, hyl, ihx, ihy;
+  float dt, lam_hi, lam_lo;              // lam = dt / (hx hy)
+  float tT, dtT;                         // t / T and dt / T (swirl)
+};
+GeoF make_geof(double x0, double y0, double hx, double hy, double t, double dt, double Tper);
+
 // Geometry and step of one problem of a batch (device array); replaces the StepParams fields of
 // the same names for the elements of that problem.
 struct ProbGeom {
@@ -119,6 +128,7 @@ struct ProbGeom {
   double x0, hx, y0, hy;
   double ghost, t, dt;
   int64_t gbase;                         // global index of the problem's first element
+  GeoF f;
 };
 
 // Element map of a 2D launch of the general kernels.  A uniform single-problem mesh uses the
@@ -184,25 +194,25 @@ struct Mixed2DExtra {
   int linref;                            // 1: linear element reference (no energy row), 0: constant
   int64_t plane;                         // float offset of the lo plane
   float span;                            // 1 / (2 (xi_{n-1} - xi_0)): corner differences to slopes
-  float hx, hy, ihx, ihy;
+  GeoF f;                                // geometry and step (a batch reads its problems' own)
   float a, b, om, cx, cy;                // velocity parameters (constant / rotation)
-  float tT, dtT;                         // t / T and dt / T (swirl)
-  float dt, dt_area;                     // dt and dt / (hx hy)
-  float lam_hi, lam_lo;                  // dt / (hx hy) as float-float
-  double Tper;                           // swirl period T (per-problem t / T in a batch), else 0
 };
 struct Work2M {                          // mixed workspace between the two phases
   float* psihat;                         // same layout as the state (one plane)
   float* traces;                         // [nel][tstride]
   float* faces;                          // [nel][4][6]  G_hi, G_lo (outflow flux of phi), U_out, U_in, P1, P2
   float* elem;                           // [nel][8]     r0, gx, gy, sum w psi, sum w psi^2, M^n hi, lo, unused
+  uint8_t* side;                         // [nel][tstride]  upwind side of each face point at t^{n+1} (see Work2D)
 };
 // per_sm: resident CTAs per SM of the persistent grid (0: as many as the occupancy allows)
 void launch_step2d_mixed(int phase, int n, const StepParams& p, const Mixed2DExtra& x, const Map2D& m,
                          int64_t count, const float* in, float* out, const Work2M& w, unsigned* status,
                          cudaStream_t s, int per_sm);
-inline int64_t work2m_floats(int64_t nel, int n) { return nel * (int64_t)(n * n + 4 * n + 24 + 8); }
 constexpr int WORK2M_FACE = 24, WORK2M_ELEM = 8;   // floats per element of the face and element records
+// floats of the workspace for nvals values and nel elements of ts face points (sides: one byte each)
+inline int64_t work2m_floats(int64_t nvals, int64_t nel, int ts) {
+  return nvals + nel * (ts + WORK2M_FACE + WORK2M_ELEM) + (nel * ts + 3) / 4;
+}
 
 // Parameters of the 2D shared-operator kernel (uniform mesh, constant velocity).  Operators that
 // every thread applies with the same entry live here (the kernel reads them from the parameter
