@@ -363,6 +363,11 @@ struct sl_ctx {
   uint16_t* d_prob = nullptr;
   sl::ProbGeom* d_geo = nullptr;
   int* d_list = nullptr;                 // element lists of the node-count buckets
+  // the buckets of a phase run side by side: on the context's stream and on these, which start after the
+  // work before the phase and are joined before the next one
+  static constexpr int NSIDE = 3;
+  cudaStream_t side[NSIDE] = {};
+  cudaEvent_t side_ev[NSIDE + 1] = {};   // fork, then one join per side stream
   // sl_run: steps captured into a CUDA graph on an internal stream, kept for identical calls
   cudaStream_t run_stream = nullptr;
   cudaEvent_t run_ev[2] = {};
