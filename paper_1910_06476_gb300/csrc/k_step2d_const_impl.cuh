@@ -27,9 +27,12 @@
 // pseudo-inverse therefore is s_F = alpha_F r + Q c_F with Q an orthonormal basis of that span (three
 // columns) and 13 coefficients per element, linear in r: about 18 products per row instead of 8 n.
 //
-// Measured (one GB300): 512 x 512 elements of n = 9, boundary and mass rows: 228 -> 192 us per step (16 bytes per
-// node take 50 us at the measured copy rate; issue 49 %, shared-memory pipe 58 % of their peaks, the rest barriers);
-// pairing the elements alone left it at 234 us, the shared-memory pipe taking the operator tables.
+// Measured (one GB300): 512 x 512 elements of n = 9, boundary and mass rows: 228 -> 182 us per step (16 bytes per
+// node take 50 us at the measured copy rate; the shared-memory pipe, barriers and issue are what is left).
+// Pairing the elements alone left it at 234 us, the shared-memory pipe taking the operator tables; the
+// structure of the pseudo-inverse and the exchanged traces made it 189; the sums between the phases spread over
+// all threads (one float-float sum of written and old mass instead of two, LN lanes an element) and four CTAs
+// per SM instead of three, 182.
 //
 // With the mass row, the element's mass target is also formed in float-float: M^n (float-float sum of
 // w (x) w (hi + lo)) minus its outflow fluxes through the x- and y-outflow faces plus its upwind
@@ -62,7 +65,10 @@ struct Tile {
   static constexpr int NR = NN | 1;               // row stride of the remapped rows
   static constexpr int PS = NN * NR + ((NN - NN * NR) & 15);   // and the stride of a pair: NN modulo 16 (same reason)
   static constexpr int PH = NP + TX / 2;          // pairs that are remapped: own and y-halo
-  static constexpr int MINB = NT <= 160 ? 4 : 3;  // resident CTAs asked of the compiler
+  // resident CTAs asked of the compiler: 72 registers up to n = 9 and 80 up to n = 11, which spill two words at
+  // most (512 x 512, n = 9: 188 -> 182 us, n = 8: 170 -> 154; 300 x 300, n = 11: 112 -> 108); 96 at n = 12 (125 us,
+  // 131 at 80 registers)
+  static constexpr int MINB = NN <= 9 ? (910 / NT > 8 ? 8 : 910 / NT) : NN <= 11 ? 819 / NT : 4;
 };
 
 // Operators applied with the same entry by every thread, each entry twice (parameter bank)
@@ -93,9 +99,9 @@ struct __align__(16) Smem {
     } f;                                          // the fit, after it
   } a;
   float2 u[T::PT * NN], v[T::PT * NN];            // outflow traces along x (before R_y) and y (relative to the own ref)
-  float2 fp[5][T::PT * NN];                       // row shares: mass residual, x and y flux, -M^n hi, lo
+  float2 fp[3][T::PT * NN];                       // row shares: mass residual, x and y flux
   float2 dx[T::NP * NN];
-  float ref[2 * T::PT], tot[3][2 * T::PT], mnh[2 * T::NP], mnl[2 * T::NP], miss[2 * T::NP];
+  float ref[2 * T::PT], tot[3][2 * T::PT], miss[2 * T::NP];
   int64_t a0[TY + 1];                             // first aligned global float of each staged row
   int off[TY + 1], nv[TY + 1];                    // row data offset in its buffer; vectors (0: gather)
 };
@@ -201,6 +207,7 @@ __global__ void __launch_bounds__(Tile<NN, TX, TY>::NT, Tile<NN, TX, TY>::MINB)
 
   // ---- row phase: thread j holds row j of psi
   float2 tau = dup(0.0f);
+  ff2 mrow = {dup(0.0f), dup(0.0f)};              // minus the row's share of M^n
   if (valid) {
     float2 q[NN];
     const float2 mref = make_float2(-ref.x, -ref.y);
@@ -231,11 +238,7 @@ __global__ void __launch_bounds__(Tile<NN, TX, TY>::NT, Tile<NN, TX, TY>::MINB)
       S.fp[0][pj] = kd;
       S.fp[1][pj] = fx;
       S.fp[2][pj] = fy;
-      if (massf) {
-        const ff2 m = mn.get();
-        S.fp[3][pj] = m.hi;
-        S.fp[4][pj] = m.lo;
-      }
+      mrow = mn.get();
     }
     if (j == 0) {
       S.ref[2 * p] = ref.x;
@@ -297,30 +300,16 @@ __global__ void __launch_bounds__(Tile<NN, TX, TY>::NT, Tile<NN, TX, TY>::MINB)
                                   gx1 ? 0.0f : us[((xn1 >> 1) * NN + j) * 2 + (xn1 & 1)]);
     S.dx[pj] = sub2(__fadd2_rn(un, drx), tau);
   }
-  // element totals of the row shares, one thread per element, rows in order (the same sums whichever CTA
-  // forms them): mass residual, outflow fluxes, M^n in float-float
+  // element totals of the row shares, one thread per element and quantity, rows in order (the same sums
+  // whichever CTA forms them): mass residual, outflow fluxes
   if (P.mass)
-    for (int e = tid; e < 2 * T::PT; e += NT) {
-      const float* f = reinterpret_cast<const float*>(S.fp) + (e >> 1) * NN * 2 + (e & 1);
-      constexpr int F = T::PT * NN * 2;
-      float kd = 0.0f, fx = 0.0f, fy = 0.0f;
+    for (int i = tid; i < 6 * T::PT; i += NT) {
+      const int q = i / (2 * T::PT), e = i - q * (2 * T::PT);
+      const float* f = reinterpret_cast<const float*>(S.fp[q]) + (e >> 1) * NN * 2 + (e & 1);
+      float v = 0.0f;
 #pragma unroll
-      for (int r = 0; r < NN; ++r) {
-        kd += f[2 * r];
-        fx += f[F + 2 * r];
-        fy += f[2 * F + 2 * r];
-      }
-      S.tot[0][e] = kd;
-      S.tot[1][e] = fx;
-      S.tot[2][e] = fy;
-      if (P.refine && e < 2 * NP) {
-        ff mn = ff_mul(ff{f[3 * F], f[4 * F]}, ff{U.wh[0].x, U.wl[0].x});
-#pragma unroll
-        for (int r = 1; r < NN; ++r)
-          mn = ff_add(mn, ff_mul(ff{f[3 * F + 2 * r], f[4 * F + 2 * r]}, ff{U.wh[r].x, U.wl[r].x}));
-        S.mnh[e] = mn.hi;
-        S.mnl[e] = mn.lo;
-      }
+      for (int r = 0; r < NN; ++r) v += f[2 * r];
+      S.tot[q][e] = v;
     }
   __syncthreads();
 
@@ -400,22 +389,28 @@ __global__ void __launch_bounds__(Tile<NN, TX, TY>::NT, Tile<NN, TX, TY>::MINB)
       if (P.refine) mv.add(U.wh[k], U.nwh[k], U.wl[k], vh[k], vl[k]);    // (column sum)
     }
     if (P.refine) {
-      const ff2 m = mv.get();
+      // minus the written column's mass plus the row's share of M^n, times their common weight w_j
+      const ff2 mc = mv.get(), m = ff_mul2(ff_add2(mc, ff2{neg2(mrow.hi), neg2(mrow.lo)}), U.wh[j], U.wl[j]);
       S.a.f.mv[0][pj] = m.hi;
       S.a.f.mv[1][pj] = m.lo;
     }
   }
   if (P.refine) {
-    // the float-float miss of the written element mass against the target, one thread per element:
+    // the float-float miss of the written element mass against the target, LN lanes per element:
     // F(element) = ref sum(f) + its total, own fluxes with this element's reference, upwind fluxes with the
     // neighbour's (or the ghost value)
     __syncthreads();
-    for (int e = tid; e < 2 * NP; e += NT) {
+    constexpr int LN = NN > 6 ? 4 : NN > 4 ? 2 : 1;
+    for (int i = tid; i < ((2 * NP * LN + 31) & ~31); i += NT) {
+      const int e = min(i / LN, 2 * NP - 1);
       const float* f = reinterpret_cast<const float*>(S.a.f.mv) + (e >> 1) * NN * 2 + (e & 1);
       constexpr int F = NP * NN * 2;
-      ff m = ff_mul(ff{f[0], f[F]}, ff{U.wh[0].x, U.wl[0].x});
+      ff m = {0.0f, 0.0f};
 #pragma unroll
-      for (int r = 1; r < NN; ++r) m = ff_add(m, ff_mul(ff{f[2 * r], f[F + 2 * r]}, ff{U.wh[r].x, U.wl[r].x}));
+      for (int q = 0; q < (NN + LN - 1) / LN; ++q) {
+        const int r = LN * q + i % LN;
+        if (r < NN) m = q == 0 ? ff{f[2 * r], f[F + 2 * r]} : ff_add(m, ff{f[2 * r], f[F + 2 * r]});
+      }
       const int x = 2 * ((e >> 1) / TY) + (e & 1), y = (e >> 1) % TY;
       const int xh = 2 * NP + y;
       const int xn = P.xw ? (x > 0 ? slot_of(x - 1, y) : xh) : (x + 1 < TX ? slot_of(x + 1, y) : xh);
@@ -426,8 +421,11 @@ __global__ void __launch_bounds__(Tile<NN, TX, TY>::NT, Tile<NN, TX, TY>::MINB)
       const float Fxu = gx ? P.gh * P.sfx : fmaf(S.ref[xn], P.sfx, S.tot[1][xn]);
       const float Fyu = gyy ? P.gh * P.sfy : fmaf(S.ref[yn], P.sfy, S.tot[2][yn]);
       // M^{n+1} = M^n - (outflow) + (inflow), float-float
-      const ff tg = ff_add(ff{-S.mnh[e], -S.mnl[e]}, ff_add(two_sum(-Fxo, -Fyo), two_sum(Fxu, Fyu)));
-      S.miss[e] = ff_to_f(ff_add(tg, m));          // (m: minus the written mass)
+      const ff fl = ff_add(two_sum(-Fxo, -Fyo), two_sum(Fxu, Fyu));
+#pragma unroll
+      for (int o = 1; o < LN; o <<= 1)
+        m = ff_add(m, ff{__shfl_xor_sync(0xffffffffu, m.hi, o), __shfl_xor_sync(0xffffffffu, m.lo, o)});
+      if (i % LN == 0 && i < 2 * NP * LN) S.miss[e] = ff_to_f(ff_add(fl, m));
     }
     __syncthreads();
     if (own) {
