@@ -99,10 +99,10 @@ struct Shape {
   // row stride of the preconditioner tables: the rows that lanes read side by side, as 16-byte vectors, start
   // in different banks
   static constexpr int RP = NP + (NP % 8 == 0 ? 4 : 0);
-  // resident CTAs asked of the compiler.  Phase 1 at three (80 registers) spills: the large swirl took 17.0 ms
-  // instead of 15.4; below two, n >= 13 ran 6-8 warps per SM.  Phase 2 fits four since the far-neighbour
-  // interpolation is out of line
-  static constexpr int MINB = 2;
+  // resident CTAs asked of the compiler.  Phase 1 at three (80 registers) fits up to n = 5 (558 / 504 us at n = 4,
+  // 4.2 M nodes) and spills above (179 / 191 us at n = 8); four CTAs of five warps at n = 17 (474 / 420 us); below
+  // two, n >= 13 ran 6-8 warps per SM.  Phase 2 fits four since the far-neighbour interpolation is out of line
+  static constexpr int MINB = NN <= 5 ? 3 : G <= 4 ? 2 : 4;
   static constexpr int MINB2 = NN <= 16 ? 4 : 3;
 };
 
@@ -641,15 +641,15 @@ __device__ __forceinline__ float dot_rows(const float* a, const float* b) {
   return r;
 }
 
-// the element of launch-list index k, and its problem's record (batches, else null)
-template <int NN>
+// the element of launch-list index k, and its problem's record (GEO: batches, else null)
+template <int NN, bool GEO>
 __device__ __forceinline__ Elem elem_at(const StepParams& P, const Map2D& M, int64_t k, const ProbGeom*& geo) {
   Elem E;
   E.g = M.list ? (int64_t)M.list[k] : k;
   E.gb = 0;
   geo = nullptr;
   int kx = P.kx;
-  if (M.geo) {
+  if (GEO) {
     geo = M.geo + M.prob[E.g];
     kx = geo->kx;
     E.gb = geo->gbase;
@@ -663,7 +663,6 @@ __device__ __forceinline__ Elem elem_at(const StepParams& P, const Map2D& M, int
 
 // a problem's mesh and float parameters into P and X (batches)
 __device__ __forceinline__ void use_problem(const ProbGeom* G, StepParams& P, Mixed2DExtra& X) {
-  if (!G) return;
   P.kx = G->kx;
   P.ky = G->ky;
   for (int f = 0; f < 4; ++f) P.bc[f] = G->bc[f];
@@ -768,7 +767,7 @@ struct Smem1 {
   float sth[2][ND], stl[2][ND];                // staged input state (hi, lo) of this and the next element
 };
 
-template <int NN>
+template <int NN, bool GEO>
 __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB)
     k_p1(StepParams P0, const __grid_constant__ Mixed2DExtra X0, Map2D M, int64_t count, const float* __restrict__ in,
          Work2M W, unsigned* status) {
@@ -799,7 +798,7 @@ __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB)
   // w (x) w at the thread's nodes as float-float
   const float2 w2h = make_float2(v0 ? X0.w2h[p0] : 0.0f, v1 ? X0.w2h[p1] : 0.0f);
   const float2 w2l = make_float2(v0 ? X0.w2l[p0] : 0.0f, v1 ? X0.w2l[p1] : 0.0f);
-  unsigned long long c_it = 0, c_floor = 0, c_nc = 0, c_feet = 0;
+  unsigned c_it = 0, c_floor = 0, c_nc = 0, c_feet = 0;
   unsigned bits = 0;
   const int64_t ngroups = (int64_t)gridDim.x * EPC;
   // asynchronous copies of element kk's input state into staging buffer b (one group per call); the element
@@ -807,7 +806,7 @@ __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB)
   auto stage = [&](int64_t kk, int b) {
     if (kk < count) {
       const ProbGeom* gn;
-      const Elem En = elem_at<NN>(P0, M, kk, gn);
+      const Elem En = elem_at<NN, GEO>(P0, M, kk, gn);
       if (t == 0) {
         sm.el[b] = En;
         sm.geo[b] = gn;
@@ -824,7 +823,7 @@ __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB)
     const Elem E = sm.el[b];
     StepParams P = P0;
     Mixed2DExtra X = X0;
-    use_problem(sm.geo[b], P, X);
+    if (GEO) use_problem(sm.geo[b], P, X);
     stage(k + ngroups, b ^ 1);
     cp_async_wait1();
     const int ex = E.ex, ey = E.ey;
@@ -853,7 +852,21 @@ __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB)
     if (v1) sm.psi[j1 * NP + i1] = pn1;
     const ff2 mn2 = ff_mul2(ff2{hi2, lo2}, w2h, w2l);
     const ff mn = ff_add(ff{mn2.hi.x, mn2.lo.x}, ff{mn2.hi.y, mn2.lo.y});
+    // element sums of psi^n (reference measure) and the float-float element mass
+    const float w20 = v0 ? s_w[i0] * s_w[j0] : 0.0f, w21 = v1 ? s_w[i1] * s_w[j1] : 0.0f;
+    float m1 = fmaf(w20, pn0, w21 * pn1), m2 = fmaf(w20 * pn0, pn0, w21 * pn1 * pn1);
     g.sync();
+    const ff Mn = g.ffsum_sum2(mn, m1, m2);
+    float* el = W.elem + E.g * 8;
+    if (t == 0) {
+      el[0] = r0;
+      el[1] = gx;
+      el[2] = gy;
+      el[3] = m1;
+      el[4] = m2;
+      el[5] = Mn.hi;
+      el[6] = Mn.lo;
+    }
     // advect the particles of nodes p0, p1 in reference coordinates
     float2 d2x = bc2(0.0f), d2y = bc2(0.0f);
     rk_disp2(V, P.rk, make_float2(s_xi[i0], s_xi[i1]), make_float2(s_xi[j0], s_xi[j1]),
@@ -928,7 +941,7 @@ __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB)
       g.sync();
       precond(false);
     }
-    c_it += (unsigned long long)(it < SOLVE_CAP ? it + 1 : SOLVE_CAP);
+    c_it += it < SOLVE_CAP ? it + 1 : SOLVE_CAP;
     if (!done) {
       // stalled, diverging or at the cap: the better of the last and the best iterate
       float acc_r = rmax;
@@ -950,20 +963,6 @@ __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB)
     }
     if (v0) W.psihat[E.base + p0] = sm.ph[j0 * NP + i0];
     if (v1) W.psihat[E.base + p1] = sm.ph[j1 * NP + i1];
-    // element sums of psi^n (reference measure) and the float-float element mass
-    const float w20 = v0 ? s_w[i0] * s_w[j0] : 0.0f, w21 = v1 ? s_w[i1] * s_w[j1] : 0.0f;
-    float m1 = fmaf(w20, pn0, w21 * pn1), m2 = fmaf(w20 * pn0, pn0, w21 * pn1 * pn1);
-    const ff Mn = g.ffsum_sum2(mn, m1, m2);
-    float* el = W.elem + E.g * 8;
-    if (t == 0) {
-      el[0] = r0;
-      el[1] = gx;
-      el[2] = gy;
-      el[3] = m1;
-      el[4] = m2;
-      el[5] = Mn.hi;
-      el[6] = Mn.lo;
-    }
     // interface values at the face points (relative to L): traces of psihat, or phi^n at the
     // backward characteristic foot of the face point from t^{n+1} (eq. 4.11; meshes of one node
     // count), L(foot) - L(face point) being the linear part over the foot's displacement
@@ -1153,7 +1152,7 @@ __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB)
       else pass1(std::false_type{}, std::false_type{});
       g.sync();
       const int nitems = sm.nitems;
-      c_feet += (unsigned long long)nitems;
+      c_feet += nitems;
       for (int it2 = t; it2 < nitems; it2 += GT) {
         const int code = sm.u.fc.items[it2];
         const int idx = code >> 2, s = code & 3;
@@ -1224,10 +1223,10 @@ __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB)
     }
   }
   if (t == 0 && X0.counts) {
-    atomicAdd(X0.counts + SL_CNT_SOLVE_ITERS, c_it);
-    if (c_floor) atomicAdd(X0.counts + SL_CNT_SOLVE_FLOOR, c_floor);
-    if (c_nc) atomicAdd(X0.counts + SL_CNT_SOLVE_NOCONV, c_nc);
-    if (c_feet) atomicAdd(X0.counts + SL_CNT_FEET, c_feet);
+    atomicAdd(X0.counts + SL_CNT_SOLVE_ITERS, (unsigned long long)c_it);
+    if (c_floor) atomicAdd(X0.counts + SL_CNT_SOLVE_FLOOR, (unsigned long long)c_floor);
+    if (c_nc) atomicAdd(X0.counts + SL_CNT_SOLVE_NOCONV, (unsigned long long)c_nc);
+    if (c_feet) atomicAdd(X0.counts + SL_CNT_FEET, (unsigned long long)c_feet);
   }
   if (bits) atomicOr(status, bits);
 }
@@ -1251,7 +1250,7 @@ struct Smem2 {
   float scal[8];
 };
 
-template <int NN>
+template <int NN, bool GEO>
 __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB2)
     k_p2(StepParams P0, const __grid_constant__ Mixed2DExtra X0, Map2D M, int64_t count, const float* __restrict__ in,
          Work2M W, float* __restrict__ out, unsigned* status) {
@@ -1286,16 +1285,16 @@ __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB2)
   const bool v0 = p0 < ND, v1 = p1 < ND;
   const int i0 = p0 % NN, j0 = (p0 / NN) % NN, i1 = p1 % NN, j1 = (p1 / NN) % NN;
   const float w20 = v0 ? s_w[i0] * s_w[j0] : 0.0f, w21 = v1 ? s_w[i1] * s_w[j1] : 0.0f;
-  unsigned long long c_el = 0, c_eapp = 0, c_pit = 0, c_pnc = 0;
+  unsigned c_el = 0, c_eapp = 0, c_pit = 0, c_pnc = 0;
   unsigned bits = 0;
   const int64_t ngroups = (int64_t)gridDim.x * EPC;
   for (int64_t k = (int64_t)blockIdx.x * EPC + g.slot; k < count; k += ngroups) {
     g.sync();
     StepParams P = P0;
     const ProbGeom* geo;
-    const Elem E = elem_at<NN>(P0, M, k, geo);
+    const Elem E = elem_at<NN, GEO>(P0, M, k, geo);
     Mixed2DExtra X = X0;
-    use_problem(geo, P, X);
+    if (GEO) use_problem(geo, P, X);
     const int ex = E.ex, ey = E.ey;
     // every global read of the element first, so that they share one memory round trip: own
     // record, psihat, input (energy), face-point traces and the neighbours' records and faces
@@ -1539,7 +1538,7 @@ __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB2)
           c21 = nv1;
           if (delta <= tol) { conv = feasible; break; }
         }
-        c_pit += (unsigned long long)(it < P.picard_cap ? it + 1 : P.picard_cap);
+        c_pit += it < P.picard_cap ? it + 1 : P.picard_cap;
         if (conv) {                                 // else keep the linear-constraint solution
           cur0 = c20 * usc;
           cur1 = c21 * usc;
@@ -1587,31 +1586,40 @@ __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB2)
     }
   }
   if (t == 0 && X0.counts) {
-    atomicAdd(X0.counts + SL_CNT_ELEMS, c_el);
-    if (c_eapp) atomicAdd(X0.counts + SL_CNT_ENERGY_APPLIED, c_eapp);
-    if (c_pit) atomicAdd(X0.counts + SL_CNT_PICARD_ITERS, c_pit);
-    if (c_pnc) atomicAdd(X0.counts + SL_CNT_PICARD_NOCONV, c_pnc);
+    atomicAdd(X0.counts + SL_CNT_ELEMS, (unsigned long long)c_el);
+    if (c_eapp) atomicAdd(X0.counts + SL_CNT_ENERGY_APPLIED, (unsigned long long)c_eapp);
+    if (c_pit) atomicAdd(X0.counts + SL_CNT_PICARD_ITERS, (unsigned long long)c_pit);
+    if (c_pnc) atomicAdd(X0.counts + SL_CNT_PICARD_NOCONV, (unsigned long long)c_pnc);
   }
   if (bits) atomicOr(status, bits);
 }
 
 // persistent grid: the resident CTAs of the whole GPU, or one CTA per EPC elements if fewer
-template <int NN>
-void launch_n(int phase, const StepParams& p, const Mixed2DExtra& x, const Map2D& m, int64_t count, const float* in,
+template <int NN, bool GEO>
+void launch_g(int phase, const StepParams& p, const Mixed2DExtra& x, const Map2D& m, int64_t count, const float* in,
               float* out, const Work2M& w, unsigned* st, cudaStream_t s, int per_sm) {
   if (count <= 0) return;
   using S = Shape<NN>;
   // phase 2 stages the fit operator for the largest row set (4 n + 1 rows), whatever p.m is, so
   // that one occupancy figure serves every launch
   const size_t smem2 = (size_t)(4 * NN + 1) * S::GT * sizeof(float2);
-  const void* kern = phase == 1 ? (const void*)k_p1<NN> : (const void*)k_p2<NN>;
+  const void* kern = phase == 1 ? (const void*)k_p1<NN, GEO> : (const void*)k_p2<NN, GEO>;
   int fill = persistent_grid(kern, S::NT, phase == 1 ? 0 : smem2);
   // per_sm > 0: that many resident CTAs per SM (the autotuner's choice), within the occupancy
   if (per_sm > 0) fill = std::min(fill, per_sm * sm_count());
   const int64_t want = (count + S::EPC - 1) / S::EPC;
   const unsigned grid = (unsigned)(want < fill ? want : fill);
-  if (phase == 1) k_p1<NN><<<grid, S::NT, 0, s>>>(p, x, m, count, in, w, st);
-  else k_p2<NN><<<grid, S::NT, smem2, s>>>(p, x, m, count, in, w, out, st);
+  if (phase == 1) k_p1<NN, GEO><<<grid, S::NT, 0, s>>>(p, x, m, count, in, w, st);
+  else k_p2<NN, GEO><<<grid, S::NT, smem2, s>>>(p, x, m, count, in, w, out, st);
+}
+
+// Batches read their problem's parameters per element; other launches have them in the parameter bank, which
+// frees about 25 registers of each kernel (256 x 256 elements of n = 8: 187 -> 179 us and 187 -> 182 us)
+template <int NN>
+void launch_n(int phase, const StepParams& p, const Mixed2DExtra& x, const Map2D& m, int64_t count, const float* in,
+              float* out, const Work2M& w, unsigned* st, cudaStream_t s, int per_sm) {
+  if (m.geo) launch_g<NN, true>(phase, p, x, m, count, in, out, w, st, s, per_sm);
+  else launch_g<NN, false>(phase, p, x, m, count, in, out, w, st, s, per_sm);
 }
 
 }  // namespace k2m
