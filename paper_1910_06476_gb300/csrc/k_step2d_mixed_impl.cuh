@@ -428,7 +428,7 @@ __device__ __forceinline__ void rk_disp(const VelElem& V, int rk, float bx, floa
 
 // vel_at at two points at once (paired float operations; the direct evaluation per component)
 __device__ __forceinline__ void vel_at2(const VelElem& V, float2 bx, float2 by, float2 Sx, float2 Cx, float2 Sy,
-                                        float2 Cy, float2 dx, float2 dy, float ct, float2& u, float2& v) {
+                                        float2 Cy, float2 dx, float2 dy, float2 ct, float2& u, float2& v) {
   switch (V.kind) {
     case SL_VEL_ROTATION: {
       const float2 x = fma2(bc2(V.hx), add2(bx, dx), bc2(V.x0)), y = fma2(bc2(V.hy), add2(by, dy), bc2(V.y0));
@@ -452,8 +452,8 @@ __device__ __forceinline__ void vel_at2(const VelElem& V, float2 bx, float2 by, 
         sy = fma2(Sy, ctt, mul2(Cy, st));
         cy = fma2(Cy, ctt, mul2(neg2(Sy), st));
       }
-      u = mul2(mul2(sx, sx), mul2(mul2(sy, cy), bc2(2.0f * ct * V.ihx)));
-      v = mul2(mul2(sy, sy), mul2(mul2(sx, cx), bc2(-2.0f * ct * V.ihy)));
+      u = mul2(mul2(sx, sx), mul2(mul2(sy, cy), mul2(ct, bc2(2.0f * V.ihx))));
+      v = mul2(mul2(sy, sy), mul2(mul2(sx, cx), mul2(ct, bc2(-2.0f * V.ihy))));
       break;
     }
     default:
@@ -462,10 +462,11 @@ __device__ __forceinline__ void vel_at2(const VelElem& V, float2 bx, float2 by, 
   }
 }
 
-// rk_disp for two points at once (paired float operations)
-template <int RK, bool TAB>
+// rk_disp for two points at once (paired float operations); cts(c) gives cos(pi tau / T) at the step fraction c of
+// each point's own step h
+template <int RK, bool TAB, class CT>
 __device__ __forceinline__ void rk_disp2_t(const VelElem& V, float2 bx, float2 by, float2 Sx, float2 Cx, float2 Sy,
-                                           float2 Cy, float2& dx, float2& dy, float h, const float* ctab) {
+                                           float2 Cy, float2& dx, float2& dy, float2 h, CT cts) {
   using T = Tab<RK>;
   float2 kx[T::S], ky[T::S];
 #pragma unroll
@@ -474,15 +475,15 @@ __device__ __forceinline__ void rk_disp2_t(const VelElem& V, float2 bx, float2 b
 #pragma unroll
     for (int j = 0; j < s; ++j)
       if (T::a(s, j) != 0.0f) {
-        const float2 hj = bc2(h * T::a(s, j));
+        const float2 hj = mul2(h, bc2(T::a(s, j)));
         xs = fma2(hj, kx[j], xs);
         ys = fma2(hj, ky[j], ys);
       }
-    const float ct = ctab[__float2int_rn(4.0f * T::c(s))];
+    const float2 ct = cts(T::c(s));
     if (TAB && s == 0) {
       const float2 p = mul2(Sx, Sy);
-      kx[0] = mul2(mul2(p, bc2(2.0f * ct * V.ihx)), mul2(Sx, Cy));
-      ky[0] = mul2(mul2(p, bc2(-2.0f * ct * V.ihy)), mul2(Sy, Cx));
+      kx[0] = mul2(mul2(p, mul2(ct, bc2(2.0f * V.ihx))), mul2(Sx, Cy));
+      ky[0] = mul2(mul2(p, mul2(ct, bc2(-2.0f * V.ihy))), mul2(Sy, Cx));
     } else if (TAB) {
       float2 st, ctt;
       small_sincos2(mul2(bc2(V.pihx), xs), V.shortser, st, ctt);
@@ -490,8 +491,8 @@ __device__ __forceinline__ void rk_disp2_t(const VelElem& V, float2 bx, float2 b
       small_sincos2(mul2(bc2(V.pihy), ys), V.shortser, st, ctt);
       const float2 sy = fma2(Sy, ctt, mul2(Cy, st)), cy = fma2(Cy, ctt, mul2(neg2(Sy), st));
       const float2 p = mul2(sx, sy);
-      kx[s] = mul2(mul2(p, bc2(2.0f * ct * V.ihx)), mul2(sx, cy));
-      ky[s] = mul2(mul2(p, bc2(-2.0f * ct * V.ihy)), mul2(sy, cx));
+      kx[s] = mul2(mul2(p, mul2(ct, bc2(2.0f * V.ihx))), mul2(sx, cy));
+      ky[s] = mul2(mul2(p, mul2(ct, bc2(-2.0f * V.ihy))), mul2(sy, cx));
     } else {
       vel_at2(V, bx, by, Sx, Cx, Sy, Cy, xs, ys, ct, kx[s], ky[s]);
     }
@@ -502,22 +503,22 @@ __device__ __forceinline__ void rk_disp2_t(const VelElem& V, float2 bx, float2 b
     sx = fma2(bc2(T::b(s)), kx[s], sx);
     sy = fma2(bc2(T::b(s)), ky[s], sy);
   }
-  dx = mul2(bc2(h), sx);
-  dy = mul2(bc2(h), sy);
+  dx = mul2(h, sx);
+  dy = mul2(h, sy);
 }
 
-// forward step over the whole step h = dt from t^n
+template <class CT>
 __device__ __forceinline__ void rk_disp2(const VelElem& V, int rk, float2 bx, float2 by, float2 Sx, float2 Cx,
-                                         float2 Sy, float2 Cy, float2& dx, float2& dy, float h, const float* ctab) {
+                                         float2 Sy, float2 Cy, float2& dx, float2& dy, float2 h, CT cts) {
   if (rk == 4 && V.kind == SL_VEL_SWIRL && !V.direct) {
-    rk_disp2_t<4, true>(V, bx, by, Sx, Cx, Sy, Cy, dx, dy, h, ctab);
+    rk_disp2_t<4, true>(V, bx, by, Sx, Cx, Sy, Cy, dx, dy, h, cts);
     return;
   }
   switch (rk) {
-    case 4: rk_disp2_t<4, false>(V, bx, by, Sx, Cx, Sy, Cy, dx, dy, h, ctab); break;
-    case 3: rk_disp2_t<3, false>(V, bx, by, Sx, Cx, Sy, Cy, dx, dy, h, ctab); break;
-    case 2: rk_disp2_t<2, false>(V, bx, by, Sx, Cx, Sy, Cy, dx, dy, h, ctab); break;
-    default: rk_disp2_t<1, false>(V, bx, by, Sx, Cx, Sy, Cy, dx, dy, h, ctab);
+    case 4: rk_disp2_t<4, false>(V, bx, by, Sx, Cx, Sy, Cy, dx, dy, h, cts); break;
+    case 3: rk_disp2_t<3, false>(V, bx, by, Sx, Cx, Sy, Cy, dx, dy, h, cts); break;
+    case 2: rk_disp2_t<2, false>(V, bx, by, Sx, Cx, Sy, Cy, dx, dy, h, cts); break;
+    default: rk_disp2_t<1, false>(V, bx, by, Sx, Cx, Sy, Cy, dx, dy, h, cts);
   }
 }
 
@@ -871,8 +872,8 @@ __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB)
     float2 d2x = bc2(0.0f), d2y = bc2(0.0f);
     rk_disp2(V, P.rk, make_float2(s_xi[i0], s_xi[i1]), make_float2(s_xi[j0], s_xi[j1]),
              make_float2(sm.T.n[0][i0], sm.T.n[0][i1]), make_float2(sm.T.n[1][i0], sm.T.n[1][i1]),
-             make_float2(sm.T.n[2][j0], sm.T.n[2][j1]), make_float2(sm.T.n[3][j0], sm.T.n[3][j1]), d2x, d2y, X.f.dt,
-             sm.T.ct);
+             make_float2(sm.T.n[2][j0], sm.T.n[2][j1]), make_float2(sm.T.n[3][j0], sm.T.n[3][j1]), d2x, d2y, bc2(X.f.dt),
+             [&](float c) { return bc2(sm.T.ct[__float2int_rn(4.0f * c)]); });
     const float dx0 = v0 ? d2x.x : 0.0f, dy0 = v0 ? d2y.x : 0.0f, dx1 = v1 ? d2x.y : 0.0f, dy1 = v1 ? d2y.y : 0.0f;
     float2 Lx[NN], Ly[NN];
     basis_at2<NN>(s_xi, s_lam, s_xi[i0], s_xi[i1], dx0, dx1, Lx);
@@ -1018,6 +1019,11 @@ __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB)
     // the stage time t^n the outflow value itself (the trace of psi^n, no foot).  Pass 2: the outflow
     // (point, stage) pairs of later stage times, compacted into a list, one backward characteristic
     // foot each.  Every pair writes its own slot; the face sums add the slots in a fixed order.
+    // Conforming elements of at most 13 nodes under the swirl take both later feet (at most two) of a face point
+    // at once in paired operations instead, with no list: a list of more than 32 pairs cost a second round, and
+    // the list its atomics and the values' way through shared memory (phase 1 with the list / with this, 4.2 M
+    // nodes: 505 / 476 us at n = 4, 290 / 276 at n = 6, 179 / 172 at n = 8, 334 / 320 at n = 12, but 376 / 398 at
+    // n = 14, where the paired bases no longer fit the registers).
     if (flux) {
       if (t < 4) {
         // points of face t and their prefix sum (lanes 0-3 of the first warp)
@@ -1071,12 +1077,13 @@ __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB)
           }
         }
       };
+      constexpr bool PAIRED = NN <= 13;
       const bool conforming = total == 4 * NN;
       const bool tab = V.kind == SL_VEL_SWIRL && !V.direct;
       // CONF: conforming faces; TAB: the swirl from the tabulated sines (both known per element)
       auto pass1 = [&](auto conf, auto tabc) {
       constexpr bool CONF = decltype(conf)::value;
-      constexpr bool TAB = decltype(tabc)::value;
+      constexpr bool PAIR = CONF && decltype(tabc)::value && PAIRED;
       for (int idx = t; idx < total; idx += GT) {
         int f, q, nq;
         float zq, xr, yr, Sx, Cx, Sy, Cy;
@@ -1116,6 +1123,7 @@ __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB)
         // per distinct stage time: the sign of u.n, the weight; later stage times that flow out
         // are queued for their backward foot (their weight kept in fbo, 0 otherwise)
         float uo = 0.0f, ui = 0.0f, q1 = 0.0f, q2 = 0.0f;
+        float2 bo = bc2(0.0f);                     // PAIR: outflow weights of the later stage times
         for (int s = 0; s < S; ++s) {
           const float cs = c_ds_c[P.rk][s];
           const float un = ubase * sm.T.ct[__float2int_rn(4.0f * cs)];
@@ -1128,6 +1136,9 @@ __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB)
               q1 = fmaf(bw, val0, q1);
               q2 = fmaf(bw * val0, val0, q2);
             }
+          } else if (PAIR) {
+            if (s == S - 1) bo.y = out ? bw : 0.0f;          // t^{n+1} is the last one,
+            else bo.x = out ? bw : 0.0f;                     // t^{n+1/2} any other
           } else {
             sm.u.fc.fbo[f][q][s] = out ? bw : 0.0f;
             // queue the pair: one shared atomic per warp (lane order within the warp)
@@ -1142,6 +1153,30 @@ __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB)
             }
           }
         }
+        if (PAIR && (bo.x != 0.0f || bo.y != 0.0f)) {
+          c_feet += (bo.x != 0.0f) + (bo.y != 0.0f);
+          float2 fdx, fdy;
+          const float2 h = make_float2(-0.5f * X.f.dt, -X.f.dt);
+          rk_disp2(V, P.rk, bc2(xr), bc2(yr), bc2(Sx), bc2(Cx), bc2(Sy), bc2(Cy), fdx, fdy, h, [&](float c) {
+            return make_float2(sm.T.ct[2 - __float2int_rn(2.0f * c)], sm.T.ct[4 - __float2int_rn(4.0f * c)]);
+          });
+          float2 bx[NN], by[NN];
+          basis_at2<NN>(s_xi, s_lam, xr, xr, fdx.x, fdx.y, bx);
+          basis_at2<NN>(s_xi, s_lam, yr, yr, fdy.x, fdy.y, by);
+          float2 val = bc2(0.0f);
+#pragma unroll
+          for (int mm = 0; mm < NN; ++mm) val = fma2(by[mm], row_dot2<NN>(sm.psi + mm * NP, bx), val);
+          // phi - r0 = (L - r0) + psi
+          val = add2(val, fma2(bc2(gx), add2(bc2(xr - 0.5f), fdx), mul2(bc2(gy), add2(bc2(yr - 0.5f), fdy))));
+          if (bo.x != 0.0f) {
+            q1 = fmaf(bo.x, val.x, q1);
+            q2 = fmaf(bo.x * val.x, val.x, q2);
+          }
+          if (bo.y != 0.0f) {
+            q1 = fmaf(bo.y, val.y, q1);
+            q2 = fmaf(bo.y * val.y, val.y, q2);
+          }
+        }
         sm.u.fc.pt[f][q][0] = uo;
         sm.u.fc.pt[f][q][1] = ui;
         sm.u.fc.pt[f][q][2] = q1;
@@ -1151,46 +1186,48 @@ __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB)
       if (conforming && tab) pass1(std::true_type{}, std::true_type{});
       else pass1(std::false_type{}, std::false_type{});
       g.sync();
-      const int nitems = sm.nitems;
-      c_feet += nitems;
-      for (int it2 = t; it2 < nitems; it2 += GT) {
-        const int code = sm.u.fc.items[it2];
-        const int idx = code >> 2, s = code & 3;
-        int f, q, nq;
-        float zq, xr, yr, Sx, Cx, Sy, Cy;
-        if (conforming) face_point(std::true_type{}, idx, f, q, nq, zq, xr, yr, Sx, Cx, Sy, Cy);
-        else face_point(std::false_type{}, idx, f, q, nq, zq, xr, yr, Sx, Cx, Sy, Cy);
-        const float cs = c_ds_c[P.rk][s];
-        float fdx = 0.0f, fdy = 0.0f;
-        rk_disp(V, P.rk, xr, yr, Sx, Cx, Sy, Cy, fdx, fdy, -cs * X.f.dt, cs, -cs, sm.T.ct);
-        float bx[NN], by[NN];
-        basis_at<NN>(s_xi, s_lam, xr, fdx, bx);
-        basis_at<NN>(s_xi, s_lam, yr, fdy, by);
-        float val = 0.0f;
-#pragma unroll
-        for (int mm = 0; mm < NN; ++mm) val = fmaf(by[mm], row_dot<NN>(sm.psi + mm * NP, bx), val);
-        val += fmaf(gx, (xr - 0.5f) + fdx, gy * ((yr - 0.5f) + fdy));   // phi - r0 = (L - r0) + psi
-        sm.u.fc.fv[f][q][s] = val;
-      }
-      g.sync();
-      // per face point: the outflow of the later stage times, added in stage order
-      if (S > 1)
-        for (int idx = t; idx < total; idx += GT) {
-          const int f = (idx >= sm.cum[1]) + (idx >= sm.cum[2]) + (idx >= sm.cum[3]);
-          const int q = idx - sm.cum[f];
-          float q1 = sm.u.fc.pt[f][q][2], q2 = sm.u.fc.pt[f][q][3];
-          for (int s = 1; s < S; ++s) {
-            const float bo = sm.u.fc.fbo[f][q][s];
-            if (bo != 0.0f) {
-              const float v = sm.u.fc.fv[f][q][s];
-              q1 = fmaf(bo, v, q1);
-              q2 = fmaf(bo * v, v, q2);
-            }
-          }
-          sm.u.fc.pt[f][q][2] = q1;
-          sm.u.fc.pt[f][q][3] = q2;
+      if (!(PAIRED && conforming && tab)) {
+        const int nitems = sm.nitems;
+        if (t == 0) c_feet += nitems;
+        for (int it2 = t; it2 < nitems; it2 += GT) {
+          const int code = sm.u.fc.items[it2];
+          const int idx = code >> 2, s = code & 3;
+          int f, q, nq;
+          float zq, xr, yr, Sx, Cx, Sy, Cy;
+          if (conforming) face_point(std::true_type{}, idx, f, q, nq, zq, xr, yr, Sx, Cx, Sy, Cy);
+          else face_point(std::false_type{}, idx, f, q, nq, zq, xr, yr, Sx, Cx, Sy, Cy);
+          const float cs = c_ds_c[P.rk][s];
+          float fdx = 0.0f, fdy = 0.0f;
+          rk_disp(V, P.rk, xr, yr, Sx, Cx, Sy, Cy, fdx, fdy, -cs * X.f.dt, cs, -cs, sm.T.ct);
+          float bx[NN], by[NN];
+          basis_at<NN>(s_xi, s_lam, xr, fdx, bx);
+          basis_at<NN>(s_xi, s_lam, yr, fdy, by);
+          float val = 0.0f;
+  #pragma unroll
+          for (int mm = 0; mm < NN; ++mm) val = fmaf(by[mm], row_dot<NN>(sm.psi + mm * NP, bx), val);
+          val += fmaf(gx, (xr - 0.5f) + fdx, gy * ((yr - 0.5f) + fdy));   // phi - r0 = (L - r0) + psi
+          sm.u.fc.fv[f][q][s] = val;
         }
-      g.sync();
+        g.sync();
+        // per face point: the outflow of the later stage times, added in stage order
+        if (S > 1)
+          for (int idx = t; idx < total; idx += GT) {
+            const int f = (idx >= sm.cum[1]) + (idx >= sm.cum[2]) + (idx >= sm.cum[3]);
+            const int q = idx - sm.cum[f];
+            float q1 = sm.u.fc.pt[f][q][2], q2 = sm.u.fc.pt[f][q][3];
+            for (int s = 1; s < S; ++s) {
+              const float bo = sm.u.fc.fbo[f][q][s];
+              if (bo != 0.0f) {
+                const float v = sm.u.fc.fv[f][q][s];
+                q1 = fmaf(bo, v, q1);
+                q2 = fmaf(bo * v, v, q2);
+              }
+            }
+            sm.u.fc.pt[f][q][2] = q1;
+            sm.u.fc.pt[f][q][3] = q2;
+          }
+        g.sync();
+      }
       // per face and quantity (16 threads): the sum over the face's points in point order
       if (t < 16) {
         const int f = t >> 2, c = t & 3;
@@ -1226,8 +1263,9 @@ __global__ void __launch_bounds__(Shape<NN>::NT, Shape<NN>::MINB)
     atomicAdd(X0.counts + SL_CNT_SOLVE_ITERS, (unsigned long long)c_it);
     if (c_floor) atomicAdd(X0.counts + SL_CNT_SOLVE_FLOOR, (unsigned long long)c_floor);
     if (c_nc) atomicAdd(X0.counts + SL_CNT_SOLVE_NOCONV, (unsigned long long)c_nc);
-    if (c_feet) atomicAdd(X0.counts + SL_CNT_FEET, (unsigned long long)c_feet);
   }
+  c_feet = __reduce_add_sync(0xffffffffu, c_feet);
+  if (g.lane == 0 && c_feet && X0.counts) atomicAdd(X0.counts + SL_CNT_FEET, (unsigned long long)c_feet);
   if (bits) atomicOr(status, bits);
 }
 

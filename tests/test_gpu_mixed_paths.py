@@ -1,6 +1,7 @@
 """Mixed-precision shared-operator kernels, which advance two elements per thread, at the sizes where their pairs,
 tiles and halos are partial: element counts around half a tile and a tile in 1D, every remainder of the tile in
-2D, both signs of the velocity, periodic and inflow faces.  Bound: 1e-6 relative L2 against the oracle, the mixed
+2D, both signs of the velocity, periodic and inflow faces; and the general kernels' face feet, taken in pairs up to
+13 nodes and from a list above and on nonconforming meshes.  Bound: 1e-6 relative L2 against the oracle, the mixed
 path's bound after one step; global mass on a periodic mesh to 1e-12 relative over 20 steps."""
 import numpy as np
 import pytest
@@ -87,3 +88,26 @@ def test_mass_over_partial_tiles(sl, dim):
     out = ctx.run(a, ctx.new_state(), gv, 0.0, dt, 20, sl.options(3, 4))
     assert ctx.sync() == 0
     assert abs(ctx.mass(out) / m0 - 1.0) <= 1e-12
+
+
+@pytest.mark.parametrize("rk", [1, 2, 3, 4])
+@pytest.mark.parametrize("n", [3, 4, 8, 9, 13, 14])
+@pytest.mark.parametrize("when", [0.3, "reversal"])
+def test_2d_face_feet_of_the_swirl(sl, n, rk, when):
+    """Every RK order's distinct stage times, and a step over which the flow reverses, so that a face point flows
+    out at some of them only; the mass row carries the face fluxes into the result."""
+    kx, ky, box = 5, 4, (0.0, 1.0, 0.0, 1.0)
+    ctx = sl.Context(2, kx, ky, box, n, 0, sl.MIXED, (1,) * 4, 0.3)
+    setup = O.Setup(2, kx, ky, box, n, 0, (1,) * 4, 0.3)
+    x, y = ctx.node_coords()
+    phi = 1.0 + 0.5 * np.sin(2 * np.pi * x) * np.cos(2 * np.pi * y) + 0.1 * np.cos(4 * np.pi * y)
+    gv = sl.velocity(sl.VEL_SWIRL, 5.0)
+    dt = ctx.max_dt(gv)
+    t = 2.5 - 0.3 * dt if when == "reversal" else when
+    src = ctx.pack(torch.tensor(phi.ravel(), device="cuda"))
+    dst = ctx.new_state()
+    ctx.step(src, dst, gv, t, dt, sl.options(sl.C_BOUNDARY | sl.C_MASS, rk))
+    assert ctx.sync() == 0
+    got = ctx.unpack(dst).cpu().numpy().reshape(phi.shape)
+    ref, _ = O.step_2d(setup, phi, O.StepOpts(O.Vel(sl.VEL_SWIRL, (5.0, 0, 0, 0, 0, 0)), t, dt, 3, rk))
+    assert rel(got, ref) <= TOL
