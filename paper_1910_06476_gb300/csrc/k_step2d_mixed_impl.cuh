@@ -38,9 +38,9 @@
 // while h <= 1/4, so that |pi h d| <= pi / 4 where ten terms are exact to 1e-9; coarser meshes evaluate
 // sinpi and cospi directly).  cos(pi t / T) is taken once per element at the stage-time fractions 0,
 // 1/4, 1/2, 3/4, 1 of the step, which cover the RK schemes and their backward feet.
-// Bound by instruction issue (63 % / 70 % of the issue slots in the two phases; FMA pipe 40 % / 30 %, HBM 4 %).
-// Measured (one GB300), 512 x 512 elements of n = 8, swirl, every constraint: phase 1 757 -> 699 us (607 -> 544 M
-// warp instructions), phase 2 597 -> 365 us (353 -> 236 M).  What that took: no FP64 instruction (element corners
+// Bound by instruction issue (60 % / 73 % of the issue slots in the two phases; FMA pipe 51 % / 32 %, HBM 4 %).
+// Measured (one GB300), 512 x 512 elements of n = 8, swirl, every constraint: phase 1 757 -> 651 us (607 -> 473 M
+// warp instructions), phase 2 597 -> 357 us (353 -> 225 M).  What that took: no FP64 instruction (element corners
 // in float-float, per-problem parameters from the host), the upwind side of each face point formed once in
 // phase 1 from the tabulated sines, the pseudo-inverse read as pairs with a thread's two nodes side by side and
 // skipped for faces whose residual vanishes, one evaluation for all tabulated sines, maxima by one integer
