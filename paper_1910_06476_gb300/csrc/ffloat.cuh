@@ -58,6 +58,11 @@ struct ff2 {
   float2 hi, lo;
 };
 __device__ __forceinline__ float2 dup(float a) { return make_float2(a, a); }
+// a stored value that is the same in both lanes
+struct fdup {
+  float v;
+  __device__ __forceinline__ operator float2() const { return make_float2(v, v); }
+};
 __device__ __forceinline__ float2 neg2(float2 a) { return make_float2(-a.x, -a.y); }
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, dup(-1.0f), a); }
 __device__ __forceinline__ ff2 two_sum2(float2 a, float2 b) {

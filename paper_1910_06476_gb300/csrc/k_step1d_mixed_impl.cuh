@@ -24,8 +24,11 @@
 //     element mass is moved along the pseudo-inverse column of the mass row into the lo words, so
 //     that the element mass meets its target to about 1e-16 relative.
 // Measured (one GB300): K = 2^20, n = 9, every constraint: 41.0 -> 37.2 us per step (16 bytes per node take
-// 22 us at the measured copy rate); 34.5 M -> 23 M warp instructions, issue 59 %, FMA pipe 54 % busy.  Five
-// CTAs per SM spill registers (42.9 us).
+// 22 us at the measured copy rate); 34.5 M -> 23 M warp instructions, issue 60 %, FMA pipe 56 % busy.  Five
+// CTAs per SM spill registers (42.9 us); from n = 14 on three CTAs with a few spills beat two without (n = 14: 58
+// against 72 us).  The operators stand in the parameter bank as single floats, duplicated into both lanes where
+// they are used: stored twice they cost every launch a cold read of up to 8 KB more (K = 4096, n = 12: 6.0 / 5.6
+// us; K = 2^20, n = 17: 79.5 / 69.3).
 // The kernel is persistent: a CTA advances tiles of TILE elements, one thread per two elements.  A
 // tile's rows (its elements and the upwind halo element) are one contiguous run of each plane;
 // one thread moves both runs into shared memory with bulk asynchronous copies (TMA) that complete
@@ -135,8 +138,8 @@ __device__ __forceinline__ TileGeo tile_geo(int K, int left_up, int t) {
 // Operators applied with the same entry by every thread, each entry twice (one per lane), and the scalars
 template <int NN>
 struct Par {
-  float2 Gs[NN * NN], rout[NN], ui[NN], um[NN];
-  float2 w[NN], E[3][NN], C[MMAX1D * NN], Cp[NN * MMAX1D], Ff[NN], wh[NN], nwh[NN], wl[NN], cmass[NN];   // nwh = -wh
+  fdup Gs[NN * NN], rout[NN], ui[NN], um[NN];
+  fdup w[NN], E[3][NN], C[MMAX1D * NN], Cp[NN * MMAX1D], Ff[NN], wh[NN], nwh[NN], wl[NN], cmass[NN];   // nwh = -wh
   float fb[3];
   int K, left_up, periodic, m, mass_on, energy_on, nst, refine, picard_cap;
   int64_t plane;
@@ -161,11 +164,11 @@ __device__ __forceinline__ void halo_row(const Par<NN>& P, const float* hi, cons
 #pragma unroll
   for (int i = 0; i < NN; ++i) {
     const float v = __fadd_rn(__fadd_rn(hi[i], -ref), lo[i]);
-    t = fmaf(P.rout[i].x, v, t);
-    f = fmaf(P.Ff[i].x, v, f);
+    t = fmaf(P.rout[i].v, v, t);
+    f = fmaf(P.Ff[i].v, v, f);
 #pragma unroll
     for (int s = 0; s < 3; ++s)
-      if (s < P.nst) e[s] = fmaf(P.E[s][i].x, v, e[s]);
+      if (s < P.nst) e[s] = fmaf(P.E[s][i].v, v, e[s]);
     mx = fmaxf(mx, fabsf(v));
   }
   X.T[row] = t;
@@ -394,7 +397,7 @@ __device__ __forceinline__ void element_step(const Par<NN>& P, Exch& X, const fl
 }
 
 template <int NN>
-__global__ void __launch_bounds__(NT, NN <= 9 ? 4 : NN <= 13 ? 3 : 2)
+__global__ void __launch_bounds__(NT, NN <= 9 ? 4 : 3)
     k_step1d_mixed(const __grid_constant__ Par<NN> P, const float* __restrict__ in, float* __restrict__ out,
                    unsigned* status) {
   constexpr int SF = stage_floats<NN>();
@@ -547,8 +550,8 @@ void launch_n(const Mixed1DParams& p, const float* in, float* out, unsigned* st,
   const int cached_grid = persistent_grid((const void*)k_step1d_mixed<NN>, NT, smem);
   const int ntiles = (p.K + TILE - 1) / TILE;
   Par<NN> P;
-  auto two = [](float2* dst, const float* src, int n) {
-    for (int i = 0; i < n; ++i) dst[i] = make_float2(src[i], src[i]);
+  auto two = [](fdup* dst, const float* src, int n) {
+    for (int i = 0; i < n; ++i) dst[i] = fdup{src[i]};
   };
   two(P.Gs, p.Gs, NN * NN);
   two(P.rout, p.rout, NN);
@@ -561,11 +564,11 @@ void launch_n(const Mixed1DParams& p, const float* in, float* out, unsigned* st,
   }
   two(P.C, p.C, MMAX1D * NN);
   for (int j = 0; j < NN; ++j)                 // rows of the pseudo-inverse at a fixed stride
-    for (int k = 0; k < MMAX1D; ++k) P.Cp[j * MMAX1D + k] = k < p.m ? make_float2(p.Cp[j * p.m + k], p.Cp[j * p.m + k]) : make_float2(0.0f, 0.0f);
+    for (int k = 0; k < MMAX1D; ++k) P.Cp[j * MMAX1D + k] = fdup{k < p.m ? p.Cp[j * p.m + k] : 0.0f};
   two(P.Ff, p.Ff, NN);
   two(P.wh, p.wh, NN);
   two(P.wl, p.wl, NN);
-  for (int i = 0; i < NN; ++i) P.nwh[i] = make_float2(-p.wh[i], -p.wh[i]);
+  for (int i = 0; i < NN; ++i) P.nwh[i] = fdup{-p.wh[i]};
   two(P.cmass, p.cmass, NN);
   P.K = p.K;
   P.left_up = p.left_up;
