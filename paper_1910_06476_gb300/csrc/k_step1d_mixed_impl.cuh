@@ -135,7 +135,7 @@ __device__ __forceinline__ TileGeo tile_geo(int K, int left_up, int t) {
   return g;
 }
 
-// Operators applied with the same entry by every thread, each entry twice (one per lane), and the scalars
+// Operators applied with the same entry by every thread (duplicated into both lanes at their use), and the scalars
 template <int NN>
 struct Par {
   fdup Gs[NN * NN], rout[NN], ui[NN], um[NN];
