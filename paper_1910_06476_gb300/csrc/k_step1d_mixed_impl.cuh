@@ -23,7 +23,7 @@
 //     neighbour, so global mass telescopes); after the fit, the float-float miss of the written
 //     element mass is moved along the pseudo-inverse column of the mass row into the lo words, so
 //     that the element mass meets its target to about 1e-16 relative.
-// Measured (one GB300): K = 2^20, n = 9, every constraint: 41.0 -> 37.2 us per step (16 bytes per node take
+// Measured (one GB300): K = 2^20, n = 9, every constraint: 41.0 -> 36.8 us per step (16 bytes per node take
 // 22 us at the measured copy rate); 34.5 M -> 23 M warp instructions, issue 60 %, FMA pipe 56 % busy.  Five
 // CTAs per SM spill registers (42.9 us); from n = 14 on three CTAs with a few spills beat two without (n = 14: 58
 // against 72 us).  The operators stand in the parameter bank as single floats, duplicated into both lanes where
